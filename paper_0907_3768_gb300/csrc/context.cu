@@ -308,7 +308,7 @@ int build_context(dust_ctx *ctx, const double *lambda, const double *w, const do
     size_t o_Ch = take(sizeof(float) * (size_t)G8 * Kp);
     size_t o_q = take(sizeof(int) * Kp);
     size_t o_w = take(sizeof(double) * K);
-    size_t o_wq = take(sizeof(float) * K);
+    size_t o_wq = take(sizeof(float) * Kp);  // zero past K
     size_t o_st = take(sizeof(int));
     DUST_CUDA_TRY(cudaMalloc(&ctx->tables_mem, off));
     ctx->tables_bytes = off;
@@ -604,7 +604,7 @@ extern "C" int dust_ctx_set_grain_numbers(dust_ctx *ctx, const double *n_g) {
     size_t off = 0;
     auto take = [&](size_t b) { const size_t o = off; off = align256(off + b); return o; };
     const size_t o_Ch = take(sizeof(float) * (size_t)G8 * Kp), o_q = take(sizeof(int) * Kp),
-                 o_wq = take(sizeof(float) * K), o_ng = take(sizeof(float) * G8), o_nax = take(sizeof(float) * Kp);
+                 o_wq = take(sizeof(float) * Kp), o_ng = take(sizeof(float) * G8), o_nax = take(sizeof(float) * Kp);
     int rc = DUST_OK;
     DevBuf t_lam, t_C;
     cudaError_t e = cudaDeviceSynchronize();
@@ -633,12 +633,12 @@ extern "C" int dust_ctx_set_grain_numbers(dust_ctx *ctx, const double *n_g) {
         double mx = 0.0;
         for (int k = 0; k < K; ++k) mx = std::max(mx, ctx->w_h[k] * std::ldexp(1.0, q[k]));
         const int Ew = mx > 0.0 ? (int)std::ceil(std::log2(mx)) : 0;
-        std::vector<float> wq(K);
+        std::vector<float> wq(Kp, 0.f);
         for (int k = 0; k < K; ++k) wq[k] = (float)std::ldexp(ctx->w_h[k], q[k] - Ew);
         const int En = (int)std::ceil(std::log2(nmax));
         std::vector<float> ng(G8, 0.f);
         for (int g = 0; g < G; ++g) ng[g] = (float)std::ldexp(n_g[g], -En);
-        e = cudaMemcpy(base + o_wq, wq.data(), sizeof(float) * K, cudaMemcpyHostToDevice);
+        e = cudaMemcpy(base + o_wq, wq.data(), sizeof(float) * Kp, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy(base + o_ng, ng.data(), sizeof(float) * G8, cudaMemcpyHostToDevice);
         if (e != cudaSuccess) rc = set_error(DUST_ECUDA, "uploading the dust-mass tables: %s", cudaGetErrorString(e));
         // residual: emitted per unit mass (h + l) 2^Ew over 4 pi absorbed per unit

@@ -59,7 +59,7 @@ struct DevTables {
     const float *Chat;        // [NKG][G8][2][4] scaled emission weights (see context.cu)
     const int *qexp;          // [Kp] per-wavelength exponent of Chat
     const double *w;          // [K] quadrature weights
-    const float *wq;          // [K] w_k 2^(q_k - Ew) (residual of the scaled emission sums)
+    const float *wq;          // [Kp] w_k 2^(q_k - Ew) (residual of the scaled emission sums), 0 in the padding
     int Ew;
     float rc_hi, rc_lo;       // 2^(Ew - Eg) / (4 pi) = (rc_hi + rc_lo) 2^rc_exp, rc_hi in [1/2, 1)
     int rc_exp;

@@ -222,6 +222,7 @@ __device__ __forceinline__ void solve_row(const EmitReq &q, int64_t cell, bool v
             if (mx > 0.f && mx < INFINITY) frexpf(mx, &mc);
         }
     }
+    const Pow2 ns = pow2_pair(-mc);
     float *Trow = q.T + c * G;
     uint8_t *frow = q.flags ? q.flags + c * G : nullptr;
     float ah = 0.f, al = 0.f;  // absorbed power n 2^-m_c Pe 2^-Eg, float-float
@@ -272,7 +273,7 @@ __device__ __forceinline__ void solve_row(const EmitReq &q, int64_t cell, bool v
             for (int i = 0; i < 4; ++i) {
                 invT[i] = PAD_INV_T;
                 nn[i] = 0.f;
-                if (g0 + i < G) grain_out(tb, g0 + i, Tv[i], fl[i], sv[i], nv[i], mc, mass, rs, invT[i], nn[i], ah, al);
+                if (g0 + i < G) grain_out(tb, g0 + i, Tv[i], fl[i], sv[i], nv[i], ns, mass, rs, invT[i], nn[i], ah, al);
             }
             // pair rows are G8 (a multiple of 8) long and 16-byte aligned
             if (mass) {

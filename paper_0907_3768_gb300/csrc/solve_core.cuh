@@ -46,12 +46,16 @@ __device__ __forceinline__ float hermite(float p0, float d0, float p1, float d1,
 // Equilibrium temperatures of NB grains at once, branch-free: every lane runs
 // the table lookup on y clamped into the table, and the clamp / invalid cases
 // are selected at the end.  s: scaled absorbed power (A / P_g(T_min) = s 2^f_g).
+// Conversions between floats and the small integers here go through the
+// float's own bits (adding 2^23): the conversion instructions run on the same
+// quarter-rate pipe as the emission's ex2, and each costs its latency in a
+// chain that is all latency.
 template <int NB>
 __device__ __forceinline__ void solve_batch(const DevTables &tb, const int (&g)[NB], const float (&s)[NB],
                                             const float4 (&gq)[NB], float (&T)[NB], int (&fl)[NB]) {
-    float y[NB], ty[NB];
-    int m[NB];
+    float ty[NB];
     float4 rv[NB];
+    const float mmax = (float)(tb.NI - 2);
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
         // y = log2 s + f_g = Y0 + ly: the integer Y0 (s's exponent plus f_g,
@@ -59,21 +63,26 @@ __device__ __forceinline__ void solve_batch(const DevTables &tb, const int (&g)[
         // is good to ~2^-22 absolute
         const int bits = __float_as_int(s[i]);
         const bool pos = s[i] > 0.f;  // false for 0, negatives and NaN
-        const float Y0 = pos ? (float)(((bits >> 23) & 0xff) - 126) + gq[i].x : 0.f;
+        // exponent field - 126, exactly: (2^23 + field) - (2^23 + 126)
+        const float ef = __int_as_float(0x4b000000 | ((bits >> 23) & 0xff)) - 8388734.f;
+        const float Y0 = pos ? ef + gq[i].x : 0.f;
         const float ly = pos ? lg2_approx(__int_as_float((bits & 0x007fffff) | 0x3f000000)) : 0.f;
-        y[i] = pos ? Y0 + ly : -INFINITY;
+        const float y = pos ? Y0 + ly : -INFINITY;
         const bool bad = !(s[i] >= 0.f) || isinf(s[i]);
-        fl[i] = bad ? DUST_FLAG_INVALID : (y[i] < 0.f ? DUST_FLAG_LOW : (y[i] > gq[i].y ? DUST_FLAG_HIGH : DUST_FLAG_OK));
+        fl[i] = bad ? DUST_FLAG_INVALID : (y < 0.f ? DUST_FLAG_LOW : (y > gq[i].y ? DUST_FLAG_HIGH : DUST_FLAG_OK));
         // interval coordinate y invdy (node m at m): the product of the
         // integer part is split exactly (ah + al) and the interval offset
         // formed from the parts, so that it keeps ~2^-24 of an interval
         // instead of ~2^-24 of y invdy (a few thousand)
         const float ah = Y0 * gq[i].z, al = fmaf(Y0, gq[i].z, -ah), b = ly * gq[i].z;
-        m[i] = min(max((int)floorf(ah + b), 0), tb.NI - 2);
-        ty[i] = fminf(fmaxf(((ah - (float)m[i]) + b) + al, 0.f), 1.f);
+        // m = floor of the coordinate clamped to [0, NI - 2], by a downward-rounded sum with 2^23
+        const float fm = __fadd_rd(fminf(fmaxf(ah + b, 0.f), mmax), 8388608.f);
+        const unsigned m = (unsigned)__float_as_int(fm) & 0x7fffffu;
+        ty[i] = fminf(fmaxf(((ah - (fm - 8388608.f)) + b) + al, 0.f), 1.f);
+        // byte offset below 2^30 (G <= 512, NI <= 65536): 32-bit arithmetic
+        rv[i] = __ldg(reinterpret_cast<const float4 *>(reinterpret_cast<const char *>(tb.ivr) +
+                                                       ((unsigned)g[i] * (unsigned)(tb.NI - 1) + m) * 16u));
     }
-#pragma unroll
-    for (int i = 0; i < NB; ++i) rv[i] = __ldg(tb.ivr + (size_t)g[i] * (tb.NI - 1) + m[i]);
     // 2^x = sum_n (x ln 2)^n / n!, five terms: |x| <= 1/8 leaves < 6e-10 (tables
     // with a wider interval take ex2)
     const float L1 = 0.69314718056f, L2 = 0.24022650695f, L3 = 0.05550410866f, L4 = 0.00961812911f,
@@ -89,19 +98,21 @@ __device__ __forceinline__ void solve_batch(const DevTables &tb, const int (&g)[
         // term alone, so it carries no cancellation.
         const float d0 = rv[i].z, d1 = rv[i].w;
         const float c2 = -2.f * d0 - d1, c3 = d0 + d1;
-        float lo = 0.f, hi = 1.f, t = ty[i];
-        for (int it = 0; it < 2; ++it) {
-            const float q = (t - ty[i]) + t * (d0 + t * (c2 + t * c3));
-            const float dq = 1.f + d0 + t * (2.f * c2 + 3.f * t * c3);
-            lo = q < 0.f ? t : lo;
-            hi = q < 0.f ? hi : t;
-            const float nt = t - q * rcp_approx(dq);
-            const bool inside = nt >= lo && nt <= hi;
-            t = inside ? nt : 0.5f * (lo + hi);
-            if (inside) break;
+        float t = ty[i];
+        const float q = t * (d0 + t * (c2 + t * c3));
+        const float dq = 1.f + d0 + t * (2.f * c2 + 3.f * t * c3);
+        float nt = t - q * rcp_approx(dq);
+        const float lo = q < 0.f ? t : 0.f, hi = q < 0.f ? 1.f : t;
+        if (!(nt >= lo && nt <= hi)) {  // rare: bisect, then one more step
+            t = 0.5f * (lo + hi);
+            const float q2 = (t - ty[i]) + t * (d0 + t * (c2 + t * c3));
+            const float dq2 = 1.f + d0 + t * (2.f * c2 + 3.f * t * c3);
+            const float lo2 = q2 < 0.f ? t : lo, hi2 = q2 < 0.f ? hi : t;
+            nt = t - q2 * rcp_approx(dq2);
+            if (!(nt >= lo2 && nt <= hi2)) nt = 0.5f * (lo2 + hi2);
         }
         // T = 2^u_m 2^(tau du)
-        const float x = t * rv[i].y;
+        const float x = nt * rv[i].y;
         const float Tv = rv[i].x * (tb.wide ? ex2_approx(x)
                                             : fmaf(x, fmaf(x, fmaf(x, fmaf(x, fmaf(x, L5, L4), L3), L2), L1), 1.f));
         T[i] = fl[i] == DUST_FLAG_OK ? Tv
@@ -110,14 +121,22 @@ __device__ __forceinline__ void solve_batch(const DevTables &tb, const int (&g)[
     }
 }
 
+// A power of two 2^e, |e| <= 252, as two normal factors: x * a * b is scale2(x, e).
+struct Pow2 { float a, b; };
+__device__ __forceinline__ Pow2 pow2_pair(int e) {
+    const int e1 = e / 2, e2 = e - e1;
+    return {__int_as_float((e1 + 127) << 23), __int_as_float((e2 + 127) << 23)};
+}
+
 // Emission pair and absorbed-power term of one solved grain g < G: the
 // pair (1/T, n 2^-m_c) the emission reads, and (rs) the grain's share of the
 // cell's absorbed power sum_g n Pe 2^-Eg added to the float-float (ah, al);
 // Pe is the absorbed power of a solved grain and P_g at the clamp otherwise.
-__device__ __forceinline__ void grain_out(const DevTables &tb, int g, float T, int fl, float s, float nv, int mc,
+// ns = 2^-m_c.
+__device__ __forceinline__ void grain_out(const DevTables &tb, int g, float T, int fl, float s, float nv, Pow2 ns,
                                           bool mass, bool rs, float &invT, float &nn, float &ah, float &al) {
     invT = rcp_approx(T);
-    nn = mass ? __ldg(tb.ng + g) : scale2(nv, -mc);
+    nn = mass ? __ldg(tb.ng + g) : nv * ns.a * ns.b;
     if (rs) {
         const float4 gr = __ldg(tb.gres + g);
         const float se = fl == DUST_FLAG_OK ? s

@@ -90,6 +90,24 @@ __device__ __forceinline__ void load_pass(const EmitReq &q, int64_t cell, int gb
     }
 }
 
+// Exponent (as frexpf's) of the largest of the lanes' mx >= 0, 0 where that is
+// 0 or infinite.  Non-negative floats order as their bits do.
+__device__ __forceinline__ int warp_exponent(float mx) {
+    const float m = __int_as_float((int)__reduce_max_sync(0xffffffffu, __float_as_uint(mx)));
+    int e = 0;
+    if (m >= 1.17549435e-38f && m < INFINITY) e = (__float_as_int(m) >> 23) - 126;
+    else if (m > 0.f && m < INFINITY) frexpf(m, &e);  // subnormal
+    return e;
+}
+
+// What the fused kernel's emission needs of a solved cell beside its pairs: the
+// exponent and (dust-mass form) mantissa bits of the cell's scale, and the cell.
+struct TileRec {
+    int mc, ms_bits;
+    int64_t cell;
+};
+static_assert(sizeof(TileRec) == sizeof(CellInfo), "plan_solve_emit sizes the records");
+
 // The solve of one cell by one warp: the exponent m_c of max_g n (general
 // form) or of the cell's mass (dust-mass form), then per pass of 32 NB grains
 // the roots, T and flags to global memory, and (emission) the pairs
@@ -101,16 +119,15 @@ __device__ __forceinline__ void load_pass(const EmitReq &q, int64_t cell, int gb
 // first pass, loaded.
 // MF: the form of n when the caller knows it (0 general, 1 dust-mass), -1 to
 // read it from the request; EMIT: the emission is known to follow (the fused
-// kernel, whose launch has NB = ceil(G8 / 32), so a cell is one pass when
-// NB < NB_MAX).
-template <int NB, bool SMEM, bool TONLY = false, int MF = -1, bool EMIT = false>
+// kernel); ONE: a cell is known to be one pass.
+template <int NB, bool SMEM, bool TONLY = false, int MF = -1, bool EMIT = false, bool ONE = false>
 __device__ __forceinline__ void solve_cell(const EmitReq &q, int64_t cell, int lane, const float (&s0)[NB],
-                                           const float (&n0)[NB], float2 *spairs, CellInfo *srec,
+                                           const float (&n0)[NB], float2 *spairs, TileRec *srec,
                                            int gsm = 1 << 30, bool also_glb = false) {
     const DevTables &tb = q.tb;
     const int G = tb.G, G8 = tb.G8;
     const bool emit = EMIT || (!TONLY && (q.mode & EMIT_ON) != 0), rs = (q.mode & EMIT_RESID) != 0;
-    const bool one = (EMIT && NB < NB_MAX) || G8 <= 32 * NB;  // known at compile time in the fused kernel
+    const bool one = ONE || G8 <= 32 * NB;
     const bool mass = MF >= 0 ? MF == 1 : (q.mode & EMIT_MASS) != 0;
     int mc = 0;
     float ms = 0.f;  // dust-mass form: m_c = ms 2^mc
@@ -122,9 +139,9 @@ __device__ __forceinline__ void solve_cell(const EmitReq &q, int64_t cell, int l
         const float *nrow = q.n + cell * G;
         float mx = 0.f;
         for (int g = lane; g < G; g += 32) mx = fmaxf(mx, __ldg(nrow + g));
-        for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        if (mx > 0.f && mx < INFINITY) frexpf(mx, &mc);
+        mc = warp_exponent(mx);
     }
+    Pow2 ns = pow2_pair(-mc);
     float ah = 0.f, al = 0.f;  // absorbed power n 2^-m_c Pe 2^-Eg, float-float
     for (int gb = 0; gb < G8; gb += 32 * NB) {
         int gi[NB], fl[NB];
@@ -146,8 +163,8 @@ __device__ __forceinline__ void solve_cell(const EmitReq &q, int64_t cell, int l
             float mx = 0.f;
 #pragma unroll
             for (int i = 0; i < NB; ++i) mx = fmaxf(mx, nv[i]);
-            for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-            if (mx > 0.f && mx < INFINITY) frexpf(mx, &mc);
+            mc = warp_exponent(mx);
+            ns = pow2_pair(-mc);
         }
         solve_batch<NB>(tb, gi, s, gq, Tv, fl);
 #pragma unroll
@@ -158,7 +175,7 @@ __device__ __forceinline__ void solve_cell(const EmitReq &q, int64_t cell, int l
             if (g < G) {
                 q.T[cell * G + g] = Tv[i];
                 if (q.flags) q.flags[cell * G + g] = (uint8_t)fl[i];
-                if (!TONLY) grain_out(tb, g, Tv[i], fl[i], s[i], nv[i], mc, mass, rs, invT, nn, ah, al);
+                if (!TONLY) grain_out(tb, g, Tv[i], fl[i], s[i], nv[i], ns, mass, rs, invT, nn, ah, al);
             }
             if (emit) {
                 if (SMEM && g < gsm) {
@@ -185,7 +202,7 @@ __device__ __forceinline__ void solve_cell(const EmitReq &q, int64_t cell, int l
             ci.al = rs ? al : 0.f;
             ci.ms_bits = __float_as_int(ms);
             q.cell[cell] = ci;
-            if (SMEM) *srec = ci;
+            if (SMEM) *srec = TileRec{mc, __float_as_int(ms), cell};
         }
     }
 }
@@ -273,6 +290,12 @@ __device__ __forceinline__ float fmin_nan(float a, float b) {
     return y;
 }
 
+__device__ __forceinline__ float fmin3_nan(float a, float b, float c) {
+    float y;
+    asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
+    return y;
+}
+
 // Regimes of a group of RG grains x the item's 8 wavelengths, on the largest
 // exponent a = nax_k / T_g in it (nax_k < 0).  Below A_ZERO every
 // t = ex2.approx.ftz(a) is flushed to 0, so the group adds nothing and is
@@ -317,9 +340,8 @@ __device__ __forceinline__ void emit_item(const float *tn, const float4 *cp, int
                 nv[u] = pr.y;
             }
         }
-        float m = iT[0];
-#pragma unroll
-        for (int u = 1; u < RG; ++u) m = fmin_nan(m, iT[u]);
+        static_assert(RG == 8, "the minimum below takes eight");
+        const float m = fmin3_nan(fmin3_nan(iT[0], iT[1], iT[2]), fmin3_nan(iT[3], iT[4], iT[5]), fmin_nan(iT[6], iT[7]));
         const float amax = naxl * m;
         if (amax < A_ZERO) continue;  // every term is 0
         const float4 *cg = cp + 2 * gg0;
@@ -382,15 +404,16 @@ __device__ __forceinline__ void emit_item(const float *tn, const float4 *cp, int
     }
 }
 
-// nax pairs of k-group ikg and the largest of its eight values.
+// nax pairs of k-group ikg and the largest of its eight values: nax rises with
+// the wavelength, and its padding is below every real value.
 __device__ __forceinline__ float load_nax(const DevTables &tb, int ikg, float2 (&nax2)[4]) {
-    float l = -INFINITY;
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-        nax2[p] = __ldg(reinterpret_cast<const float2 *>(tb.nax + ikg * KQ) + p);
-        l = fmaxf(l, fmaxf(nax2[p].x, nax2[p].y));
-    }
-    return l;
+    const float4 *p = reinterpret_cast<const float4 *>(tb.nax + ikg * KQ);
+    const float4 a = __ldg(p), b = __ldg(p + 1);
+    nax2[0] = make_float2(a.x, a.y);
+    nax2[1] = make_float2(a.z, a.w);
+    nax2[2] = make_float2(b.x, b.y);
+    nax2[3] = make_float2(b.z, b.w);
+    return __ldg(tb.nax + min(ikg * KQ + KQ, tb.K) - 1);
 }
 
 // Cell of slot i of a request's emission order.
@@ -411,20 +434,17 @@ template <bool MASS>
 __device__ __forceinline__ void emit_item_out(const EmitReq &q, int64_t cell, int ikg, const float2 (&acc)[4], int mc,
                                               float ms, bool storeL, bool vecL, bool rs) {
     const DevTables &tb = q.tb;
-    const int K = tb.K;
-    float sh = 0.f, sl = 0.f;
-    const int kb = ikg * KQ;
-    float Lv[KQ];
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int k = min(kb + 2 * p + h, K - 1);
-            const float a = h ? acc[p].y : acc[p].x;
-            Lv[2 * p + h] = scale2(MASS ? a * ms : a, mc + __ldg(tb.qexp + k));
-        }
-    }
+    const int K = tb.K, kb = ikg * KQ;
+    // qexp and wq are padded to whole k-groups
     if (storeL) {
+        const int4 qa = __ldg(reinterpret_cast<const int4 *>(tb.qexp + kb)), qb = __ldg(reinterpret_cast<const int4 *>(tb.qexp + kb) + 1);
+        const int qe[KQ] = {qa.x, qa.y, qa.z, qa.w, qb.x, qb.y, qb.z, qb.w};
+        float Lv[KQ];
+#pragma unroll
+        for (int j = 0; j < KQ; ++j) {
+            const float a = j & 1 ? acc[j >> 1].y : acc[j >> 1].x;
+            Lv[j] = scale2(MASS ? a * ms : a, mc + qe[j]);
+        }
         float *row = q.L + cell * q.ld + kb;
         if (vecL && kb + KQ <= K) {
             reinterpret_cast<float4 *>(row)[0] = make_float4(Lv[0], Lv[1], Lv[2], Lv[3]);
@@ -435,20 +455,18 @@ __device__ __forceinline__ void emit_item_out(const EmitReq &q, int64_t cell, in
                 if (kb + j < K) row[j] = Lv[j];
         }
     }
+    float sh = 0.f, sl = 0.f;
     if (rs) {
+        const float4 wa = __ldg(reinterpret_cast<const float4 *>(tb.wq + kb)), wb = __ldg(reinterpret_cast<const float4 *>(tb.wq + kb) + 1);
+        const float wk[KQ] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
 #pragma unroll
-        for (int p = 0; p < 4; ++p) {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int k = kb + 2 * p + h;
-                if (k < K) {
-                    // w_k L_k 2^-(m_c + Ew) = wq_k a: the FP32 accumulator before
-                    // its power-of-two scaling (equal to the stored L unless L is subnormal)
-                    const float a = h ? acc[p].y : acc[p].x;
-                    const float wk = __ldg(tb.wq + k);
-                    const float pr = wk * a;
-                    ff_add(sh, sl, pr, fmaf(wk, a, -pr));
-                }
+        for (int j = 0; j < KQ; ++j) {
+            if (kb + j < K) {
+                // w_k L_k 2^-(m_c + Ew) = wq_k a: the FP32 accumulator before
+                // its power-of-two scaling (equal to the stored L unless L is subnormal)
+                const float a = j & 1 ? acc[j >> 1].y : acc[j >> 1].x;
+                const float pr = wk[j] * a;
+                ff_add(sh, sl, pr, fmaf(wk[j], a, -pr));
             }
         }
     }
@@ -473,8 +491,8 @@ __device__ __forceinline__ void emit_item_out(const EmitReq &q, int64_t cell, in
 // emitted once filled[b] >= i / KE_NBUF + 1, and refilled once drained[b]
 // counts every item of the tiles put there before it.  Waits poll with a
 // short sleep, are bounded, and record DUST_ETIMEOUT.
-constexpr int KE_W = 15;                // emission warps
-constexpr int KE_TH = (KE_W + 1) * 32;  // and one copier warp: 512 threads, 128 registers
+constexpr int KE_W = 23;                // emission warps (15 of 128 registers: 3 % slower)
+constexpr int KE_TH = (KE_W + 1) * 32;  // and one copier warp: 768 threads, 80 registers
 constexpr int KE_NBUF = 3;
 
 __device__ __forceinline__ void cp_async8(void *dst, const void *src) {
@@ -584,13 +602,19 @@ __global__ void __launch_bounds__(KE_TH, 1) k_emit(const __grid_constant__ EmitB
         const bool first = q.g0 == 0, last = q.g1 == G8;
         const bool rs = (q.mode & EMIT_RESID) != 0, storeL = (q.mode & EMIT_STORE_L) != 0;
         const bool vecL = storeL && ((reinterpret_cast<uintptr_t>(q.L) & 15) == 0) && (q.ld % 4 == 0);
-        for (;;) {
+        int i = 0, rem = 0;  // the claimed item: tile of the unit, item in it
+        {
             int w = 0;
             if (lane == 0) w = atomicAdd(claim, 1);
-            w = __shfl_sync(0xffffffffu, w, 0);
-            const int i = w / NKG;
+            rem = __shfl_sync(0xffffffffu, w, 0);
+        }
+        for (;;) {
+            for (; rem >= NKG; rem -= NKG) ++i;
             if (i >= ntl) break;
-            const int ikg = NKG - 1 - (w - i * NKG);
+            // the next item is claimed now, so that the counter's latency hides behind this one
+            int w = 0;
+            if (lane == 0) w = atomicAdd(claim, 1);
+            const int ikg = NKG - 1 - rem;
             const int b = i % KE_NBUF;
             if (!warp_wait_geq(&filled[b], i / KE_NBUF + 1, abort_flag, tb.status, lane)) break;
             const int64_t c0 = (t0 + i) * TC;
@@ -616,6 +640,7 @@ __global__ void __launch_bounds__(KE_TH, 1) k_emit(const __grid_constant__ EmitB
             }
             __syncwarp();
             if (lane == 0) add_release_cta(&drained[b], 1);
+            rem = __shfl_sync(0xffffffffu, w, 0) - i * NKG;
         }
     }
 }
@@ -653,30 +678,39 @@ __device__ __forceinline__ void cell_resid(const EmitReq &q, int64_t cell) {
 // wait is bounded, and on expiry the kernel records DUST_ETIMEOUT and both
 // roles wind down.  Buffer phases: a warp waits on full[b] for tile ti only
 // once that buffer's previous tile (ti - FSE_NBUF) is filled.  Claims run in
-// order and each emission warp holds at most one unfinished item, so with
-// fewer than NKG (FSE_NBUF - 1) emission warps active, a claim in tile ti
-// implies a finished item in tiles ti - FSE_NBUF + 1 .. ti - 1, hence (tiles
-// are filled in order) a filled tile ti - FSE_NBUF.  The kernel keeps the
-// active emission warps below that bound.
-constexpr int FE_W = 12;  // emission warps
-constexpr int FS_W = 8;   // solver warps
-constexpr int FSE_TH = (FE_W + FS_W) * 32;  // 640 threads: 96 registers each
+// order and each emission warp holds at most two unfinished items (the one it
+// emits and the one it has claimed ahead), so with at most NKG (FSE_NBUF - 1) / 2
+// emission warps active, an item of tile ti implies a finished item among the
+// NKG FSE_NBUF items of tiles ti - FSE_NBUF .. ti - 1, hence (tiles are filled
+// in order) a filled tile ti - FSE_NBUF.  The kernel keeps the active emission
+// warps below that bound.
+// Emission and solver warps: 24 of 80 registers each (six per SM
+// sub-partition).  Both roles are bound by the latency of their own
+// instructions, not by a pipe, so warps count more than registers: 262144
+// cells x 200 x 96 took 0.88 ms with 12 + 8 warps of 96 registers and 0.84 ms
+// with these, once claims, tile numbers and tables no longer stood in the
+// items' way (0.91 ms before); without any solve 12, 16 and 20 emission warps
+// take 0.74, 0.70 and 0.69 ms, and fewer than 8 solver warps fall behind.
+constexpr int fe_w(bool pass) { return pass ? 12 : 16; }
+constexpr int fs_w(bool pass) { return pass ? 12 : 8; }
+constexpr int fse_th(bool pass) { return (fe_w(pass) + fs_w(pass)) * 32; }
 constexpr int FSE_NBUF = 3;  // pair-tile buffers: the solvers run up to FSE_NBUF tiles ahead
 constexpr int FSE_TC = 32;   // cells per tile: one per lane of an emission item
 
-// The CTA's it-th tile.  Its tiles are blockIdx.x + j gridDim.x, coldest
+// The CTA's it-th tile.  Its nb tiles are blockIdx.x + j gridDim.x, coldest
 // cells first (the emission order); they are taken from both ends in turn
 // (first, last, second, second to last, ...), so that tiles of cheap
 // emission (cold cells: many groups skipped) alternate with expensive ones
-// and the solve, whose cost per tile is even, stays in step.
-__device__ __forceinline__ int64_t fse_tile(int64_t it, int64_t ntiles) {
-    const int64_t nb = (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x;  // this CTA's tiles
-    const int64_t j = (it & 1) ? nb - 1 - (it >> 1) : (it >> 1);
-    return it < nb ? blockIdx.x + j * gridDim.x : ntiles;
+// and the solve, whose cost per tile is even, stays in step.  Tiles are
+// counted in 32 bits (the emission order's cell numbers are).
+__device__ __forceinline__ int fse_tile(int it, int nb) {
+    const int j = (it & 1) ? nb - 1 - (it >> 1) : (it >> 1);
+    return (int)blockIdx.x + j * (int)gridDim.x;
 }
 
 template <int NB, bool MASS, bool PASS>
-__global__ void __launch_bounds__(FSE_TH, 1) k_solve_emit(const __grid_constant__ EmitReq q) {
+__global__ void __launch_bounds__(fse_th(PASS), 1) k_solve_emit(const __grid_constant__ EmitReq q) {
+    constexpr int FE_W = fe_w(PASS), FS_W = fs_w(PASS), FSE_TH = fse_th(PASS);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const DevTables &tb = q.tb;
     const int G8 = tb.G8, NKG = tb.NKG;
@@ -692,13 +726,14 @@ __global__ void __launch_bounds__(FSE_TH, 1) k_solve_emit(const __grid_constant_
     constexpr int PW = MASS ? 1 : 2;  // floats per pair
     float4 *sC = reinterpret_cast<float4 *>(smem_raw);                          // [NKG][CST]
     float *sP = reinterpret_cast<float *>(sC + (size_t)NKG * CST);             // [FSE_NBUF][TC][PS][PW]
-    CellInfo *sI = reinterpret_cast<CellInfo *>(sP + (((size_t)FSE_NBUF * TC * PS * PW + 3) & ~(size_t)3));  // [FSE_NBUF][TC]
+    TileRec *sI = reinterpret_cast<TileRec *>(sP + (((size_t)FSE_NBUF * TC * PS * PW + 3) & ~(size_t)3));  // [FSE_NBUF][TC]
     uint64_t *full = reinterpret_cast<uint64_t *>(sI + FSE_NBUF * TC);         // [FSE_NBUF]
     uint64_t *empty = full + FSE_NBUF;                                         // [FSE_NBUF]
     volatile int *abort_flag = reinterpret_cast<volatile int *>(empty + FSE_NBUF);
     int *claim = const_cast<int *>(abort_flag) + 1;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int64_t ntiles = (q.C + TC - 1) / TC;
+    const int ntiles = (int)((q.C + TC - 1) / TC);
+    const int nb = (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;  // this CTA's tiles
 
     {
         const float4 *src = reinterpret_cast<const float4 *>(tb.Chat);
@@ -719,35 +754,39 @@ __global__ void __launch_bounds__(FSE_TH, 1) k_solve_emit(const __grid_constant_
         // ------------------------------------------------------------ solvers
         const int sw = warp - FE_W;
         const bool rs = (q.mode & EMIT_RESID) != 0 && whole;  // else the fold follows the last pass
-        int it = 0;
-        int64_t tile = fse_tile(0, ntiles);
+        // the cells of this tile's and the next one's 32 slots, a slot per lane
+        auto slots = [&](int it) -> int64_t {
+            const int64_t i = it < nb ? (int64_t)fse_tile(it, nb) * TC + lane : q.C;
+            return i < q.C ? ordered_cell(q, i) : -1;
+        };
+        int64_t cells = slots(0);
         float s0[NB], n0[NB];
-        int64_t pf = -1;  // the tile whose first slot of this warp s0 / n0 hold
+        bool have = false;  // s0 / n0 hold this warp's first slot of the tile
         bool ok = true;
-        for (; tile < ntiles && ok; tile = fse_tile(++it, ntiles)) {
+        int it = 0;
+        for (; it < nb && ok; ++it) {
             const int b = it % FSE_NBUF;
             const uint32_t ph = (uint32_t)((it / FSE_NBUF) & 1);
-            const int nc = (int)min((int64_t)TC, q.C - tile * TC);
+            const int nc = (int)min((int64_t)TC, q.C - (int64_t)fse_tile(it, nb) * TC);
+            const int64_t next = slots(it + 1);
             // a warp with no slot in the previous tile (a ragged one) prefetched nothing
-            if (sw < nc && pf != tile) load_pass<NB>(q, ordered_cell(q, tile * TC + sw), 0, lane, s0, n0);
+            if (sw < nc && !have) load_pass<NB>(q, __shfl_sync(0xffffffffu, cells, sw), 0, lane, s0, n0);
             if (!(ok = mbar_wait(&empty[b], ph ^ 1, abort_flag, tb.status))) break;
             // the buffer's previous tile (it - FSE_NBUF) is fully emitted: one
             // solver warp, in turn, folds its cells' residuals (lane = cell)
             if (rs && it >= FSE_NBUF && sw == it % FS_W) {
-                const int64_t i = fse_tile(it - FSE_NBUF, ntiles) * TC + lane;
+                const int64_t i = (int64_t)fse_tile(it - FSE_NBUF, nb) * TC + lane;
                 if (i < q.C) cell_resid(q, ordered_cell(q, i));
             }
+            have = false;
             for (int cl = sw; cl < nc; cl += FS_W) {
-                const int64_t cell = ordered_cell(q, tile * TC + cl);
+                const int64_t cell = __shfl_sync(0xffffffffu, cells, cl);
                 // next cell of this warp: in this tile, else its first in the next tile
-                int64_t tn = tile;
-                int cn = cl + FS_W;
-                if (cn >= nc) { tn = fse_tile(it + 1, ntiles); cn = sw; }
-                const bool more = tn < ntiles && tn * TC + cn < q.C;
+                const int64_t cn = cl + FS_W < nc ? __shfl_sync(0xffffffffu, cells, cl + FS_W) : __shfl_sync(0xffffffffu, next, sw);
                 float s1[NB], n1[NB];
-                if (more) load_pass<NB>(q, ordered_cell(q, tn * TC + cn), 0, lane, s1, n1);
-                pf = more ? tn : -1;
-                solve_cell<NB, true, false, MASS ? 1 : 0, true>(q, cell, lane, s0, n0,
+                have = cn >= 0;
+                if (have) load_pass<NB>(q, cn, 0, lane, s1, n1);
+                solve_cell<NB, true, false, MASS ? 1 : 0, true, !PASS && NB < NB_MAX>(q, cell, lane, s0, n0,
                                                                 reinterpret_cast<float2 *>(sP + ((size_t)b * TC + cl) * PS * PW),
                                                                 sI + b * TC + cl, PASS ? gc : 1 << 30, PASS);
 #pragma unroll
@@ -755,51 +794,57 @@ __global__ void __launch_bounds__(FSE_TH, 1) k_solve_emit(const __grid_constant_
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&full[b]);
+            cells = next;
         }
         // the residuals of the last FSE_NBUF tiles, once their emission is done
         if (rs && ok && sw == 0)
             for (int j = max(0, it - FSE_NBUF); j < it; ++j) {
                 if (!mbar_wait(&empty[j % FSE_NBUF], (uint32_t)((j / FSE_NBUF) & 1), abort_flag, tb.status)) break;
-                const int64_t i = fse_tile(j, ntiles) * TC + lane;
+                const int64_t i = (int64_t)fse_tile(j, nb) * TC + lane;
                 if (i < q.C) cell_resid(q, ordered_cell(q, i));
             }
     } else {
         // ------------------------------------------------------------ emission
-        if (warp >= NKG * (FSE_NBUF - 1) - 1) return;  // see the phase argument above
+        if (warp >= max(1, NKG * (FSE_NBUF - 1) / 2)) return;  // see the phase argument above
         const bool rs = (q.mode & EMIT_RESID) != 0, storeL = (q.mode & EMIT_STORE_L) != 0;
         const bool vecL = storeL && ((reinterpret_cast<uintptr_t>(q.L) & 15) == 0) && (q.ld % 4 == 0);
-        for (;;) {
+        int ti = 0, rem = 0;  // the claimed item: the CTA's tile and the item in it
+        {
             int w = 0;
             if (lane == 0) w = atomicAdd(claim, 1);
-            w = __shfl_sync(0xffffffffu, w, 0);
-            const int ti = w / NKG;
-            const int ikg = NKG - 1 - (w - ti * NKG);
-            const int64_t tile = fse_tile(ti, ntiles);
-            if (tile >= ntiles) break;
+            rem = __shfl_sync(0xffffffffu, w, 0);
+        }
+        for (;;) {
+            for (; rem >= NKG; rem -= NKG) ++ti;
+            if (ti >= nb) break;
+            // the next item is claimed now, so that the counter's latency hides behind this one
+            int w = 0;
+            if (lane == 0) w = atomicAdd(claim, 1);
+            const int ikg = NKG - 1 - rem;
             const int b = ti % FSE_NBUF;
             const uint32_t ph = (uint32_t)((ti / FSE_NBUF) & 1);
+            float2 nax2[4], acc[4];
+            const float naxl = load_nax(tb, ikg, nax2);
             if (!mbar_wait(&full[b], ph, abort_flag, tb.status)) break;
-            const int nc = (int)min((int64_t)TC, q.C - tile * TC);
+            const int nc = (int)min((int64_t)TC, q.C - (int64_t)fse_tile(ti, nb) * TC);
             if (lane < nc) {
-                float2 nax2[4], acc[4];
-                const float naxl = load_nax(tb, ikg, nax2);
 #pragma unroll
                 for (int p = 0; p < 4; ++p) acc[p] = make_float2(0.f, 0.f);
                 emit_item<MASS, PW>(sP + ((size_t)b * TC + lane) * PS * PW, sC + (size_t)ikg * CST, gc, nax2, naxl, acc);
-                const int64_t cell = ordered_cell(q, tile * TC + lane);
+                const TileRec tr = sI[b * TC + lane];
                 if constexpr (whole) {
-                    const CellInfo ci = sI[b * TC + lane];
-                    emit_item_out<MASS>(q, cell, ikg, acc, ci.mc, MASS ? __int_as_float(ci.ms_bits) : 1.f, storeL,
+                    emit_item_out<MASS>(q, tr.cell, ikg, acc, tr.mc, MASS ? __int_as_float(tr.ms_bits) : 1.f, storeL,
                                         vecL, rs);
                 } else {
                     // the first pass's sums, carried to the next (k_emit's layout)
-                    float2 *ap = q.accp + ((size_t)cell * NKG + ikg) * 4;
+                    float2 *ap = q.accp + ((size_t)tr.cell * NKG + ikg) * 4;
 #pragma unroll
                     for (int p = 0; p < 4; ++p) ap[p] = acc[p];
                 }
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty[b]);
+            rem = __shfl_sync(0xffffffffu, w, 0) - ti * NKG;
         }
     }
 }
@@ -1079,10 +1124,10 @@ int launch_fse(const EmitReq &r, int nb, unsigned grid, size_t smem, cudaStream_
                                : reinterpret_cast<const void *>(k_solve_emit<4, MASS, PASS>);
     DUST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     switch (nb) {
-        case 1: k_solve_emit<1, MASS, PASS><<<grid, FSE_TH, smem, st>>>(r); break;
-        case 2: k_solve_emit<2, MASS, PASS><<<grid, FSE_TH, smem, st>>>(r); break;
-        case 3: k_solve_emit<3, MASS, PASS><<<grid, FSE_TH, smem, st>>>(r); break;
-        default: k_solve_emit<4, MASS, PASS><<<grid, FSE_TH, smem, st>>>(r); break;
+        case 1: k_solve_emit<1, MASS, PASS><<<grid, fse_th(PASS), smem, st>>>(r); break;
+        case 2: k_solve_emit<2, MASS, PASS><<<grid, fse_th(PASS), smem, st>>>(r); break;
+        case 3: k_solve_emit<3, MASS, PASS><<<grid, fse_th(PASS), smem, st>>>(r); break;
+        default: k_solve_emit<4, MASS, PASS><<<grid, fse_th(PASS), smem, st>>>(r); break;
     }
     DUST_CUDA_TRY(cudaGetLastError());
     return DUST_OK;
@@ -1101,10 +1146,16 @@ int launch_solve_emit_fused(const EmitReq &req, int TC, size_t smem, int num_sms
     r.tile_begin = 0;
     E.ncells = r.C;
     E.ntiles = (r.C + TC - 1) / TC;
-    const int nb = std::min(NB_MAX, (r.tb.G8 + 31) / 32);
+    // grains per lane and pass of the solver warps: a cell is one pass up to
+    // 32 NB_MAX grains.  With grain passes the first launch solves every grain
+    // but emits only a chunk of them, so its solver warps are its critical
+    // role: more of them, and three grains per lane, where a fourth spills at
+    // their 80 registers (131072 cells x 500 x 240: 3.01 ms per step with 12 +
+    // 12 warps and three, 3.03 with four, 3.05 with 12 + 8 warps and four).
+    const bool pass = r.g1 - r.g0 < r.tb.G8;  // the first of several grain passes
+    const int nb = std::min(pass ? 3 : NB_MAX, (r.tb.G8 + 31) / 32);
     const bool mass = (r.mode & EMIT_MASS) != 0;
     const unsigned grid = (unsigned)std::min<int64_t>(E.ntiles, num_sms);
-    const bool pass = r.g1 - r.g0 < r.tb.G8;  // the first of several grain passes
     int rc = mass ? (pass ? launch_fse<true, true>(r, nb, grid, smem, st) : launch_fse<true, false>(r, nb, grid, smem, st))
                   : (pass ? launch_fse<false, true>(r, nb, grid, smem, st) : launch_fse<false, false>(r, nb, grid, smem, st));
     if (rc != DUST_OK) return rc;
