@@ -161,6 +161,14 @@ struct EmitPlan {
     size_t smem;
 };
 
+// Geometry of a small call's solve + emission: the CTAs a tile's k-groups are
+// split over (0: not a small call), lanes per cell of an emission item (tiles
+// are of 32 / lpc cells), bytes of shared memory per CTA.
+struct SplitPlan {
+    int parts, lpc;
+    size_t smem;
+};
+
 // One request of the tensor-core absorption kernel (its TMA descriptor for J
 // sits in TcBatch::tm at the same index).
 struct TcReq {
@@ -179,6 +187,8 @@ struct TcBatch {
     int GsMax, ns1, ns2, tmem_cols, nacc, off_exp, j_off;
     int orient;  // 0: cells are the MMA's M (128-cell tiles); 1: cells are its N (256-cell tiles, Gs <= 128)
     int *status;
+    int *zero;      // nzero words to clear for a later kernel of the same call (or nzero = 0)
+    int nzero;
 };
 
 // One request of the FP32 SIMT absorption kernel.
@@ -193,6 +203,8 @@ struct SimtBatch {
     SimtReq req[MAXREQ];
     int nreq;
     int64_t ntiles;
+    int *zero;      // as TcBatch's
+    int nzero;
 };
 
 }  // namespace dust
@@ -285,10 +297,12 @@ const char *cuda_err_name(cudaError_t e);
     } while (0)
 
 // Kernels' entry points (host launchers), each returning a dust_status.
+// (zero, nzero: words the absorption kernel also clears, for counters of a
+// later kernel of the call)
 int launch_gemm_simt(const dust_ctx *ctx, int64_t C, const float *J, int64_t ld, float *S,
-                     cudaStream_t st);
+                     cudaStream_t st, int *zero = nullptr, int nzero = 0);
 int launch_gemm_tc(const dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t ld,
-                   float *S, cudaStream_t st);
+                   float *S, cudaStream_t st, int *zero = nullptr, int nzero = 0);
 int launch_solve_emit(const dust_ctx *ctx, int64_t C, const ScratchView &sv, const float *n, float *T,
                       float *L, int64_t ld, double *resid, uint8_t *flags, cudaStream_t st, int *nlaunch = nullptr);
 EmitPlan plan_emit(const dust_ctx *ctx, bool emit, bool mass);
@@ -337,6 +351,11 @@ inline int order_ref_grain(int G) { return G / 2; }
 size_t plan_solve_emit(const dust_ctx *ctx, bool emit, bool mass, int *TC, int *gc);
 int launch_solve_emit_fused(const EmitReq &req, int TC, size_t smem, int num_sms, cudaStream_t st,
                             int *nlaunch = nullptr);
+
+// A small call's solve + emission with each tile's k-groups split over several
+// CTAs: the plan, and the launch (cnt: one zeroed counter per tile).
+SplitPlan plan_solve_emit_split(const dust_ctx *ctx, int64_t C, bool mass);
+int launch_solve_emit_split(const EmitReq &r, const SplitPlan &p, int *cnt, cudaStream_t st);
 
 // Grow the context's scratch to hold `cells` cells (synchronises `st` first).
 int ensure_scratch(dust_ctx *ctx, int64_t cells, cudaStream_t st);

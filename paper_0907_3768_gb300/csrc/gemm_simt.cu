@@ -22,6 +22,8 @@ __global__ void __launch_bounds__(NTH, 2) k_gemm_simt(const __grid_constant__ Si
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
 
     const int64_t tile = blockIdx.x;
+    if (tile == 0)
+        for (int i = tid; i < B.nzero; i += NTH) B.zero[i] = 0;
     int ri = 0;
     while (ri + 1 < B.nreq && tile >= B.req[ri + 1].tile_begin) ++ri;
     const SimtReq &q = B.req[ri];
@@ -162,10 +164,13 @@ int launch_simt_batch(SimtBatch &B, cudaStream_t st) {
     return DUST_OK;
 }
 
-int launch_gemm_simt(const dust_ctx *ctx, int64_t C, const float *J, int64_t ld, float *S, cudaStream_t st) {
+int launch_gemm_simt(const dust_ctx *ctx, int64_t C, const float *J, int64_t ld, float *S, cudaStream_t st,
+                     int *zero, int nzero) {
     if (C <= 0) return DUST_OK;
     SimtBatch B;
     B.nreq = 1;
+    B.zero = zero;
+    B.nzero = nzero;
     make_simt_req(ctx, C, J, ld, S, B.req[0]);
     return launch_simt_batch(B, st);
 }

@@ -100,11 +100,19 @@ int solve_view(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t 
     B.nreq = 1;
     fill_emit_req(ctx, p, C, sv, n, T, L, ld, resid, flags, B.req[0], mass);
     const bool fused = ctx->fused && precision != DUST_PREC_FP32;
+    const bool fuse_emit = !fused && ctx->fused_emit && (L || resid);
+    // small calls: tiles split over CTAs, which count their finished parts in
+    // words of the pair scratch (these kernels keep the pairs in shared
+    // memory) that the absorption kernel clears
+    const SplitPlan split = fuse_emit ? plan_solve_emit_split(ctx, C, mass) : SplitPlan{};
+    int *cnt = reinterpret_cast<int *>(sv.prep);
+    const int ncnt = split.parts > 1 && resid ? (int)((C * split.lpc + 31) / 32) : 0;
     int rc = DUST_OK;
     if (fused) {
         // one kernel through the temperatures: S stays in tensor memory
         TcBatch tb;
         tb.nreq = 1;
+        tb.nzero = 0;
         tb.status = ctx->tb.status;
         tb.orient = 0;
         SolveList sl;
@@ -114,18 +122,17 @@ int solve_view(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t 
         if (rc == DUST_OK) rc = finish_tc_batch(tb, precision, ctx->smem_optin, &smem, true);
         if (rc == DUST_OK) rc = launch_tc_batch(tb, precision, smem, ctx->num_sms, st, &sl);
     } else {
-        rc = precision == DUST_PREC_FP32 ? launch_gemm_simt(ctx, C, J, ld, sv.S, st)
-                                         : launch_gemm_tc(ctx, precision, C, J, ld, sv.S, st);
+        rc = precision == DUST_PREC_FP32 ? launch_gemm_simt(ctx, C, J, ld, sv.S, st, cnt, ncnt)
+                                         : launch_gemm_tc(ctx, precision, C, J, ld, sv.S, st, cnt, ncnt);
     }
     if (rc == DUST_OK) nl_total += 1;
     int ftc = 0, fgc = 0;
-    const size_t fsmem = !fused && ctx->fused_emit ? plan_solve_emit(ctx, L || resid, mass, &ftc, &fgc) : 0;
+    const size_t fsmem = fuse_emit && !split.parts ? plan_solve_emit(ctx, L || resid, mass, &ftc, &fgc) : 0;
     if (fsmem && fgc != p.gcp) return set_error(DUST_EINVAL, "internal: grain passes of the two emission forms differ");
     // The emission order groups cells of like temperatures into the emission's
-    // 32-cell tiles; it never changes a result.  A call of at most one tile per
-    // SM skips it: there the ordering's three launches cost more than the
-    // warp-uniform regimes save.
-    const bool ordered = C > (int64_t)32 * ctx->num_sms;
+    // 32-cell tiles; it never changes a result.  Small calls skip it: there the
+    // ordering's three launches cost more than the warp-uniform regimes save.
+    const bool ordered = !split.parts && C > (int64_t)32 * ctx->num_sms;
     if (rc == DUST_OK && (L || resid) && ordered && sv.order && sv.bkt && sv.hist) {
         // emission order: cells classed by the absorbed power of the reference
         // grain (S), or by its inverse temperature where S stayed in tensor memory
@@ -153,7 +160,11 @@ int solve_view(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t 
     if (rc == DUST_OK) {
         if (ev && ev[1]) DUST_CUDA_TRY(cudaEventRecord(ev[1], st));
         int nl = 0;
-        if (fsmem) {
+        if (split.parts) {
+            if (ev && ev[2]) DUST_CUDA_TRY(cudaEventRecord(ev[2], st));
+            rc = launch_solve_emit_split(B.req[0], split, cnt, st);
+            if (rc == DUST_OK) nl = 1;
+        } else if (fsmem) {
             // the solve runs inside the emission kernel: its time is reported with the emission's;
             // where the grains come in passes the kernel emits the first and k_emit the others
             if (ev && ev[2]) DUST_CUDA_TRY(cudaEventRecord(ev[2], st));

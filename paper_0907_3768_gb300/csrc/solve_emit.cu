@@ -118,15 +118,16 @@ static_assert(sizeof(TileRec) == sizeof(CellInfo), "plan_solve_emit sizes the re
 // also_glb the pairs of every grain to q.prep too.  s0 / n0: this cell's
 // first pass, loaded.
 // MF: the form of n when the caller knows it (0 general, 1 dust-mass), -1 to
-// read it from the request; EMIT: the emission is known to follow (the fused
+// read it from the request; store: false leaves global memory alone (another
+// CTA solves the same cell for it).  EMIT: the emission is known to follow (the fused
 // kernel); ONE: a cell is known to be one pass.
 template <int NB, bool SMEM, bool TONLY = false, int MF = -1, bool EMIT = false, bool ONE = false>
 __device__ __forceinline__ void solve_cell(const EmitReq &q, int64_t cell, int lane, const float (&s0)[NB],
                                            const float (&n0)[NB], float2 *spairs, TileRec *srec,
-                                           int gsm = 1 << 30, bool also_glb = false) {
+                                           int gsm = 1 << 30, bool also_glb = false, bool store = true) {
     const DevTables &tb = q.tb;
     const int G = tb.G, G8 = tb.G8;
-    const bool emit = EMIT || (!TONLY && (q.mode & EMIT_ON) != 0), rs = (q.mode & EMIT_RESID) != 0;
+    const bool emit = EMIT || (!TONLY && (q.mode & EMIT_ON) != 0), rs = (q.mode & EMIT_RESID) != 0 && store;
     const bool one = ONE || G8 <= 32 * NB;
     const bool mass = MF >= 0 ? MF == 1 : (q.mode & EMIT_MASS) != 0;
     int mc = 0;
@@ -173,8 +174,10 @@ __device__ __forceinline__ void solve_cell(const EmitReq &q, int64_t cell, int l
             if (g >= G8) continue;
             float invT = PAD_INV_T, nn = 0.f;
             if (g < G) {
-                q.T[cell * G + g] = Tv[i];
-                if (q.flags) q.flags[cell * G + g] = (uint8_t)fl[i];
+                if (store) {
+                    q.T[cell * G + g] = Tv[i];
+                    if (q.flags) q.flags[cell * G + g] = (uint8_t)fl[i];
+                }
                 if (!TONLY) grain_out(tb, g, Tv[i], fl[i], s[i], nv[i], ns, mass, rs, invT, nn, ah, al);
             }
             if (emit) {
@@ -201,7 +204,7 @@ __device__ __forceinline__ void solve_cell(const EmitReq &q, int64_t cell, int l
             ci.ah = rs ? ah : 0.f;
             ci.al = rs ? al : 0.f;
             ci.ms_bits = __float_as_int(ms);
-            q.cell[cell] = ci;
+            if (store) q.cell[cell] = ci;
             if (SMEM) *srec = TileRec{mc, __float_as_int(ms), cell};
         }
     }
@@ -321,21 +324,37 @@ constexpr float A_MID = -12.f;
 //   regime test is exact for every term of the group.
 // Every lane's arithmetic depends only on its own cell, so results are the
 // same in any batch, kernel or lane arrangement.
-// GLB: tn is the cell's row of the solve's scratch in global memory, read
-// through the read-only path (L1), instead of a shared-memory tile.
-template <bool MASS, int PST, bool GLB = false>
-__device__ __forceinline__ void emit_item(const float *tn, const float4 *cp, int gn, const float2 (&nax2)[4],
-                                          float naxl, float2 (&acc)[4]) {
+// NP: the wavelength pairs this lane takes of the group (4, or fewer where
+// several lanes share a cell's group, cp and nax2 being this lane's part).
+template <int NP>
+__device__ __forceinline__ void load_weights(const float4 *cg, float2 (&cw)[NP]) {
+    if constexpr (NP == 4) {
+        const float4 ca = cg[0], cb = cg[1];
+        cw[0] = make_float2(ca.x, ca.y);
+        cw[1] = make_float2(ca.z, ca.w);
+        cw[2] = make_float2(cb.x, cb.y);
+        cw[3] = make_float2(cb.z, cb.w);
+    } else if constexpr (NP == 2) {
+        const float4 ca = cg[0];
+        cw[0] = make_float2(ca.x, ca.y);
+        cw[1] = make_float2(ca.z, ca.w);
+    } else {
+        cw[0] = *reinterpret_cast<const float2 *>(cg);
+    }
+}
+
+template <bool MASS, int PST, int NP>
+__device__ __forceinline__ void emit_item(const float *tn, const float4 *cp, int gn, const float2 (&nax2)[NP],
+                                          float naxl, float2 (&acc)[NP]) {
     for (int gg0 = 0; gg0 < gn; gg0 += RG) {
         float iT[RG], nv[RG];
 #pragma unroll
         for (int u = 0; u < RG; ++u) {
             if (MASS) {
-                iT[u] = GLB ? __ldg(tn + (gg0 + u) * PST) : tn[(gg0 + u) * PST];
+                iT[u] = tn[(gg0 + u) * PST];
                 nv[u] = 0.f;
             } else {
-                const float2 *pp = reinterpret_cast<const float2 *>(tn + (gg0 + u) * PST);
-                const float2 pr = GLB ? __ldg(pp) : *pp;
+                const float2 pr = *reinterpret_cast<const float2 *>(tn + (gg0 + u) * PST);
                 iT[u] = pr.x;
                 nv[u] = pr.y;
             }
@@ -345,15 +364,14 @@ __device__ __forceinline__ void emit_item(const float *tn, const float4 *cp, int
         const float amax = naxl * m;
         if (amax < A_ZERO) continue;  // every term is 0
         const float4 *cg = cp + 2 * gg0;
+        float2 cw[NP];
         if (amax < A_WIEN) {
 #pragma unroll
             for (int u = 0; u < RG; ++u) {
-                const float4 ca = cg[2 * u], cb = cg[2 * u + 1];
-                const float2 cw[4] = {make_float2(ca.x, ca.y), make_float2(ca.z, ca.w), make_float2(cb.x, cb.y),
-                                      make_float2(cb.z, cb.w)};
+                load_weights<NP>(cg + 2 * u, cw);
                 const float2 i2 = make_float2(iT[u], iT[u]);
 #pragma unroll
-                for (int p = 0; p < 4; ++p) {
+                for (int p = 0; p < NP; ++p) {
                     const float2 a = __fmul2_rn(nax2[p], i2);
                     const float2 t = make_float2(ex2_approx(a.x), ex2_approx(a.y));
                     const float2 w = MASS ? cw[p] : __fmul2_rn(make_float2(nv[u], nv[u]), cw[p]);
@@ -363,12 +381,10 @@ __device__ __forceinline__ void emit_item(const float *tn, const float4 *cp, int
         } else if (amax < A_MID) {
 #pragma unroll
             for (int u = 0; u < RG; ++u) {
-                const float4 ca = cg[2 * u], cb = cg[2 * u + 1];
-                const float2 cw[4] = {make_float2(ca.x, ca.y), make_float2(ca.z, ca.w), make_float2(cb.x, cb.y),
-                                      make_float2(cb.z, cb.w)};
+                load_weights<NP>(cg + 2 * u, cw);
                 const float2 i2 = make_float2(iT[u], iT[u]);
 #pragma unroll
-                for (int p = 0; p < 4; ++p) {
+                for (int p = 0; p < NP; ++p) {
                     const float2 a = __fmul2_rn(nax2[p], i2);
                     const float2 t = make_float2(ex2_approx(a.x), ex2_approx(a.y));
                     const float2 w = MASS ? cw[p] : __fmul2_rn(make_float2(nv[u], nv[u]), cw[p]);
@@ -376,16 +392,14 @@ __device__ __forceinline__ void emit_item(const float *tn, const float4 *cp, int
                 }
             }
         } else {
-            float2 N[4], D[4];
+            float2 N[NP], D[NP];
 #pragma unroll
             for (int u = 0; u < RG; ++u) {
-                const float4 ca = cg[2 * u], cb = cg[2 * u + 1];
-                const float2 cw[4] = {make_float2(ca.x, ca.y), make_float2(ca.z, ca.w), make_float2(cb.x, cb.y),
-                                      make_float2(cb.z, cb.w)};
+                load_weights<NP>(cg + 2 * u, cw);
                 const float2 i2 = make_float2(iT[u], iT[u]);
                 const float2 n2 = make_float2(nv[u], nv[u]);
 #pragma unroll
-                for (int p = 0; p < 4; ++p) {
+                for (int p = 0; p < NP; ++p) {
                     if (MASS) {
                         if (u == 0) emit_first_m(nax2[p], i2, cw[p], N[p], D[p]);
                         else emit_pair_m(nax2[p], i2, cw[p], N[p], D[p]);
@@ -396,7 +410,7 @@ __device__ __forceinline__ void emit_item(const float *tn, const float4 *cp, int
                 }
             }
 #pragma unroll
-            for (int p = 0; p < 4; ++p) {
+            for (int p = 0; p < NP; ++p) {
                 acc[p].x = fmaf(N[p].x, rcp_approx(D[p].x), acc[p].x);
                 acc[p].y = fmaf(N[p].y, rcp_approx(D[p].y), acc[p].y);
             }
@@ -629,7 +643,7 @@ __global__ void __launch_bounds__(KE_TH, 1) k_emit(const __grid_constant__ EmitB
                 // the cell record is read now, so that its latency hides behind the sums
                 CellInfo ci{};
                 if (last) ci = q.cell[cell];
-                emit_item<MASS, PW>(sP + ((size_t)b * TC + lane) * PS * PW, sC + (size_t)ikg * CST, gc, nax2, naxl, acc);
+                emit_item<MASS, PW, 4>(sP + ((size_t)b * TC + lane) * PS * PW, sC + (size_t)ikg * CST, gc, nax2, naxl, acc);
                 if (last) {
                     emit_item_out<MASS>(q, cell, ikg, acc, ci.mc, MASS ? __int_as_float(ci.ms_bits) : 1.f, storeL, vecL,
                                         rs);
@@ -651,11 +665,14 @@ __device__ __forceinline__ void cell_resid(const EmitReq &q, int64_t cell) {
     const int NKG = q.tb.NKG;
     const float2 *pp = q.part + cell * NKG;
     float h = 0.f, l = 0.f;
+    // through L2: the partials may be another SM's
+#pragma unroll 8
     for (int kg = 0; kg < NKG; ++kg) {
-        const float2 v = pp[kg];
+        const float2 v = __ldcg(pp + kg);
         ff_add(h, l, v.x, v.y);
     }
-    const CellInfo ci = q.cell[cell];
+    const int4 cv = __ldcg(reinterpret_cast<const int4 *>(q.cell + cell));
+    const CellInfo ci{cv.x, __int_as_float(cv.y), __int_as_float(cv.z), cv.w};
     q.resid[cell] = (double)residual(h, l, ci.ah, ci.al, q.tb);
 }
 
@@ -830,7 +847,7 @@ __global__ void __launch_bounds__(fse_th(PASS), 1) k_solve_emit(const __grid_con
             if (lane < nc) {
 #pragma unroll
                 for (int p = 0; p < 4; ++p) acc[p] = make_float2(0.f, 0.f);
-                emit_item<MASS, PW>(sP + ((size_t)b * TC + lane) * PS * PW, sC + (size_t)ikg * CST, gc, nax2, naxl, acc);
+                emit_item<MASS, PW, 4>(sP + ((size_t)b * TC + lane) * PS * PW, sC + (size_t)ikg * CST, gc, nax2, naxl, acc);
                 const TileRec tr = sI[b * TC + lane];
                 if constexpr (whole) {
                     emit_item_out<MASS>(q, tr.cell, ikg, acc, tr.mc, MASS ? __int_as_float(tr.ms_bits) : 1.f, storeL,
@@ -847,6 +864,104 @@ __global__ void __launch_bounds__(fse_th(PASS), 1) k_solve_emit(const __grid_con
             rem = __shfl_sync(0xffffffffu, w, 0) - ti * NKG;
         }
     }
+}
+
+// Small calls: k_solve_emit's work where there are too few 32-cell tiles to
+// keep every SM at it.  In the fused kernel above such a call runs on as many
+// SMs as it has tiles, each of them loading every weight, solving its cells
+// four to a warp and then emitting 25 items (K = 200) on 16 warps in two
+// rounds, nothing of which overlaps anything.  Here a tile is 32 / LPC cells,
+// LPC (2 or 4) lanes sharing a cell's k-group (4 / LPC wavelength pairs each), and its
+// k-groups are split over `parts` CTAs: each solves the tile's cells for
+// itself (the first one stores T, flags and records), loads the weights of
+// its own k-groups only, and emits them (plan_solve_emit_split).  Every value is formed by the
+// same operations in the same order as in the fused kernel.  The residual of
+// a tile is folded by the CTA that finishes last of its parts (cnt, zeroed by
+// the absorption kernel before this one).
+constexpr int SPL_W = 12;            // warps per CTA, two CTAs per SM (80 registers)
+constexpr int SPL_TH = SPL_W * 32;
+
+template <int NB, bool MASS, int LPC>
+__global__ void __launch_bounds__(SPL_TH, 2) k_solve_emit_split(const __grid_constant__ EmitReq q, int parts, int *cnt) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int TC = FSE_TC / LPC, PW = MASS ? 1 : 2, NP = 4 / LPC;
+    const DevTables &tb = q.tb;
+    const int G8 = tb.G8, NKG = tb.NKG, CST = 2 * G8 + 1, PS = G8 + 1;
+    const int tile = blockIdx.x / parts, part = blockIdx.x - tile * parts;
+    const int k0 = part * NKG / parts, k1 = (part + 1) * NKG / parts;  // this CTA's k-groups
+    const int c0 = tile * TC, nc = (int)min((int64_t)TC, q.C - c0);
+    float4 *sC = reinterpret_cast<float4 *>(smem_raw);                  // [k1 - k0][CST]
+    float *sP = reinterpret_cast<float *>(sC + (size_t)((NKG + parts - 1) / parts) * CST);  // [TC][PS][PW]
+    TileRec *sI = reinterpret_cast<TileRec *>(sP + (((size_t)TC * PS * PW + 3) & ~(size_t)3));  // [TC]
+    int *claim = reinterpret_cast<int *>(sI + TC);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const bool rs = (q.mode & EMIT_RESID) != 0, storeL = (q.mode & EMIT_STORE_L) != 0;
+
+    // solve: warp w takes cells w, w + SPL_W, ...; the weights' loads are issued first
+    const float4 *src = reinterpret_cast<const float4 *>(tb.Chat) + (size_t)k0 * G8 * 2;
+    for (int i = tid; i < (k1 - k0) * 2 * G8; i += SPL_TH) {
+        const int kg = i / (2 * G8);
+        sC[i + kg] = __ldg(src + i);  // rows of CST = 2 G8 + 1
+    }
+    if (tid == 0) *claim = 0;
+    float s0[NB], n0[NB];
+    if (warp < nc) load_pass<NB>(q, ordered_cell(q, c0 + warp), 0, lane, s0, n0);
+    for (int cl = warp; cl < nc; cl += SPL_W) {
+        float s1[NB], n1[NB];
+        if (cl + SPL_W < nc) load_pass<NB>(q, ordered_cell(q, c0 + cl + SPL_W), 0, lane, s1, n1);
+        solve_cell<NB, true, false, MASS ? 1 : 0, true>(q, ordered_cell(q, c0 + cl), lane, s0, n0,
+                                                        reinterpret_cast<float2 *>(sP + (size_t)cl * PS * PW), sI + cl,
+                                                        1 << 30, false, part == 0);
+#pragma unroll
+        for (int i = 0; i < NB; ++i) { s0[i] = s1[i]; n0[i] = n1[i]; }
+    }
+    __syncthreads();
+
+    // emission: an item is one k-group of the tile, the longest wavelengths first
+    const bool vecL = storeL && ((reinterpret_cast<uintptr_t>(q.L) & 15) == 0) && (q.ld % 4 == 0);
+    const int sub = lane % LPC, cl = lane / LPC;
+    const bool on = cl < nc;
+    const TileRec tr = sI[on ? cl : 0];
+    for (int w = warp; w < k1 - k0;) {
+        const int ikg = k1 - 1 - w;
+        float2 nax2[NP], acc[NP];
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            nax2[p] = __ldg(reinterpret_cast<const float2 *>(tb.nax + ikg * KQ) + sub * NP + p);
+            acc[p] = make_float2(0.f, 0.f);
+        }
+        const float naxl = __ldg(tb.nax + min(ikg * KQ + KQ, tb.K) - 1);
+        if (on)
+            emit_item<MASS, PW, NP>(sP + (size_t)cl * PS * PW,
+                                    reinterpret_cast<const float4 *>(reinterpret_cast<const float2 *>(sC + (size_t)(ikg - k0) * CST) + sub * NP),
+                                    G8, nax2, naxl, acc);
+        const float ms = MASS ? __int_as_float(tr.ms_bits) : 1.f;
+        // the eight sums of the cell's k-group on every one of its lanes
+        float2 all[4];
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            all[j].x = __shfl_sync(0xffffffffu, acc[j % NP].x, lane - sub + j / NP);
+            all[j].y = __shfl_sync(0xffffffffu, acc[j % NP].y, lane - sub + j / NP);
+        }
+        if (on && sub == 0) emit_item_out<MASS>(q, tr.cell, ikg, all, tr.mc, ms, storeL, vecL, rs);
+        if (lane == 0) w = SPL_W + atomicAdd(claim, 1);
+        w = __shfl_sync(0xffffffffu, w, 0);
+    }
+    if (!rs) return;
+    // the tile's residuals, once every part's partials and part 0's records are there
+    __syncthreads();
+    if (warp != 0) return;
+    int last = 1;
+    if (parts > 1) {
+        if (lane == 0) {
+            __threadfence();
+            last = atomicAdd(cnt + tile, 1) == parts - 1;
+            __threadfence();
+        }
+        last = __shfl_sync(0xffffffffu, last, 0);
+    }
+    if (last && lane < nc) cell_resid(q, ordered_cell(q, c0 + lane));
 }
 
 // Energy-balance residual of every cell of the requests that want it: one
@@ -1131,6 +1246,62 @@ int launch_fse(const EmitReq &r, int nb, unsigned grid, size_t smem, cudaStream_
     }
     DUST_CUDA_TRY(cudaGetLastError());
     return DUST_OK;
+}
+
+// Small calls (k_solve_emit_split): lanes per cell, the parts a tile's k-groups
+// are split into and shared memory, or parts = 0 where the fused kernel takes
+// the call.
+SplitPlan plan_solve_emit_split(const dust_ctx *ctx, int64_t C, bool mass) {
+    const DevTables &tb = mass ? ctx->tbm : ctx->tb;
+    SplitPlan p{};
+    const int64_t sms = ctx->num_sms;
+    // Where the fused kernel takes over.  It needs tiles of like temperatures, so
+    // the cell ordering (three launches, 16 us), and whole tiles for every SM; a
+    // small call is emitted unordered, which costs about half as much again per
+    // term.  Times per call of the fused kernel and of this one, in us: 200 x 96,
+    // 4900 cells 73 / 66, 7000 76 / 70, 8192 77 / 86, 9728 76 / 80; 64 x 16, 9728
+    // cells 38 / 22, 12288 43 / 29; 500 x 240, 4900 cells 354 / 303, 7000 369 / 425.
+    if (C > 40 * sms && (C > 96 * sms || (double)C * tb.K * tb.G > 1.5e8)) return p;
+    // Four lanes per cell while tiles of 8 cells make at most two CTAs per SM, the
+    // most that run at once; then two.  (200 x 96, in us with 1, 2 and 4 lanes: 32
+    // cells 35 / 29 / 25, 1024 cells 39 / 35 / 31, 2048 cells 49 / 39 / 37, 4864
+    // cells 60 / 49 / 57.)
+    p.lpc = C <= 16 * sms ? 4 : 2;
+    const int tc = FSE_TC / p.lpc;
+    const int64_t tiles = (C + tc - 1) / tc;
+    auto bytes = [&](int parts) {
+        return (size_t)((tb.NKG + parts - 1) / parts) * (2 * tb.G8 + 1) * 16 +
+               (((size_t)tc * (tb.G8 + 1) * (mass ? 4 : 8) + 15) & ~(size_t)15) + tc * sizeof(TileRec) + 16;
+    };
+    // Parts only to fill the SMs once, since each repeats the solve, and to fit
+    // the weights (two CTAs per SM where the tiles are short).  500 x 240, 1024
+    // cells: 3 parts (one CTA per SM) 113 us, 6 parts 100 us.
+    const size_t budget = (ctx->smem_optin ? ctx->smem_optin : 99 * 1024) - 1024;
+    int parts = (int)std::max<int64_t>(1, std::min<int64_t>(tb.NKG, sms / tiles));
+    while (parts < tb.NKG && bytes(parts) > (p.lpc == 4 ? budget / 2 : budget)) ++parts;
+    if (bytes(parts) > budget) return p;
+    p.parts = parts;
+    p.smem = bytes(parts);
+    return p;
+}
+
+template <bool MASS, int LPC>
+int launch_split(const EmitReq &r, int nb, unsigned grid, const SplitPlan &p, int *cnt, cudaStream_t st) {
+    auto kern = nb == 1 ? k_solve_emit_split<1, MASS, LPC> : nb == 2 ? k_solve_emit_split<2, MASS, LPC>
+              : nb == 3 ? k_solve_emit_split<3, MASS, LPC> : k_solve_emit_split<4, MASS, LPC>;
+    DUST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem));
+    kern<<<grid, SPL_TH, p.smem, st>>>(r, p.parts, cnt);
+    DUST_CUDA_TRY(cudaGetLastError());
+    return DUST_OK;
+}
+
+int launch_solve_emit_split(const EmitReq &r, const SplitPlan &p, int *cnt, cudaStream_t st) {
+    const int nb = std::min(NB_MAX, (r.tb.G8 + 31) / 32);
+    const int tc = FSE_TC / p.lpc;
+    const unsigned grid = (unsigned)((r.C + tc - 1) / tc * p.parts);
+    if (r.mode & EMIT_MASS)
+        return p.lpc == 4 ? launch_split<true, 4>(r, nb, grid, p, cnt, st) : launch_split<true, 2>(r, nb, grid, p, cnt, st);
+    return p.lpc == 4 ? launch_split<false, 4>(r, nb, grid, p, cnt, st) : launch_split<false, 2>(r, nb, grid, p, cnt, st);
 }
 
 int launch_solve_emit_fused(const EmitReq &req, int TC, size_t smem, int num_sms, cudaStream_t st,
