@@ -24,9 +24,10 @@
 //   5. steady state by the balance of the probability fluxes across each cut
 //      between levels j-1 and j:  P_j = sum_{i<j} P_i Phi(j-i) / cool_j,
 //      computed forward: every new P_j adds P_j Phi(f-j) to the flux into
-//      each level f > j (the problem's lanes own the levels: a half-warp
-//      for up to 64 levels, two problems per warp, a whole warp from 128
-//      levels on), so each step is M/lanes FMAs per lane and one shuffle;
+//      each level f > j (the problem's lanes own the levels, each a run of
+//      consecutive ones: a half-warp for up to 64 levels, two problems per
+//      warp, a whole warp from 128 levels on), so each step is M/lanes FMAs
+//      per lane, two to an instruction, and one shuffle;
 //   6. emission L[c,k] = 4 pi sum_g n sum_j P_j C[g,k] B_k(T_j) (Eqs. 8-10),
 //      one MUFU ex2 per (level, wavelength), the level sum accumulated as a
 //      fraction with one reciprocal per 8 levels.
@@ -43,6 +44,7 @@
 #include "solve_core.cuh"
 
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 namespace dust {
@@ -72,10 +74,14 @@ constexpr int FL_NPL = 4;  // emission: wavelength pairs per lane per pass (256 
 
 __host__ __device__ constexpr int fl_k4(int K) { return (K + 3) & ~3; }
 __host__ __device__ constexpr int fl_kl(int K) { return (K + 255) & ~255; }
-// per-warp shared memory, every array 16-byte aligned:
-//   (1/T, P) [M] pairs, M zeros then phi [M], kb [M], x [K4], Sh [K4+4],
-//   Sf [K4+4], Lw [KL]
-__host__ __device__ constexpr size_t fl_lw_offset(int K, int M) { return (size_t)5 * M + 3 * (size_t)fl_k4(K) + 8; }
+// per-slot shared memory, every array 16-byte aligned:
+//   (1/T, P) [M] pairs, M zeros then phi [M], then kb [M], x [K4], Sh [K4+4],
+//   Sf [K4+4] while phi is formed and afterwards, in their place, M zeros then
+//   phi moved up by one [M], and Lw [KL]
+__host__ __device__ constexpr size_t fl_lw_offset(int K, int M) {
+    const size_t form = (size_t)M + 3 * (size_t)fl_k4(K) + 8, moved = (size_t)2 * M;
+    return (size_t)4 * M + (form > moved ? form : moved);
+}
 // slot stride: 16 more than a multiple of 32 floats, so that the two problems
 // of a warp (one per half) sit 16 banks apart
 __host__ __device__ constexpr size_t fl_warp_floats(int K, int M) {
@@ -153,6 +159,37 @@ __device__ __forceinline__ void fl_pass(const DevTables &tb, const float2 *LT, i
     }
 }
 
+// A lane's run of N (2 or 4) consecutive floats, and its NR runs of each N lanes' worth.
+template <int N>
+__device__ __forceinline__ void load_run(const float *p, float (&v)[N]) {
+    if constexpr (N == 2) {
+        const float2 a = *reinterpret_cast<const float2 *>(p);
+        v[0] = a.x; v[1] = a.y;
+    } else {
+        const float4 a = *reinterpret_cast<const float4 *>(p);
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    }
+}
+template <int N, int NR>
+__device__ __forceinline__ void load_runs(const float *p, int lane, int lanes, float (&v)[N * NR]) {
+#pragma unroll
+    for (int g = 0; g < NR; ++g) {
+        float t[N];
+        load_run<N>(p + N * (g * lanes + lane), t);
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[N * g + i] = t[i];
+    }
+}
+template <int N, int NR>
+__device__ __forceinline__ void store_runs(float *p, int lane, int lanes, const float (&v)[N * NR]) {
+#pragma unroll
+    for (int g = 0; g < NR; ++g) {
+        float *d = p + N * (g * lanes + lane);
+        if constexpr (N == 2) *reinterpret_cast<float2 *>(d) = make_float2(v[2 * g], v[2 * g + 1]);
+        else *reinterpret_cast<float4 *>(d) = make_float4(v[N * g], v[N * g + 1], v[N * g + 2], v[N * g + 3]);
+    }
+}
+
 // Lanes per (cell, grain) problem: 16 up to 64 levels (two problems per
 // warp, whose recursion chains overlap in one instruction stream; measured
 // 6 % faster at M = 64), 32 above (measured faster from M = 128 on, where a
@@ -175,7 +212,9 @@ __global__ void __launch_bounds__(fl_threads(M), fl_min_ctas(M)) k_fluct(const D
                                                                       float *L, float *P, float *dE_out,
                                                                       float eps_ref) {
     constexpr int LW = fl_lanes(M);
-    constexpr int MR = M / LW;    // levels per lane
+    constexpr int MR = M / LW;             // levels per lane,
+    constexpr int RN = MR < 4 ? MR : 4;    // in runs of RN consecutive ones:
+    constexpr int NR = MR / RN;            // register r is level level_of(r)
     constexpr int PPW = 32 / LW;  // problems per warp
     extern __shared__ float sm[];
     const int K = tb.K, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -183,12 +222,15 @@ __global__ void __launch_bounds__(fl_threads(M), fl_min_ctas(M)) k_fluct(const D
     const unsigned hmask = LW == 32 ? 0xffffffffu : (0xffffu << (lane & 16));
     const int64_t c = blockIdx.x;
     if (c >= C) return;
+    auto level_of = [&](int r) { return (r / RN) * (RN * LW) + RN * hl + r % RN; };
     const float inv_h2 = 1.f / tb.h2;
     const int Kp4 = (K + 3) & ~3;
     float *Jc = sm;
     float *base = sm + Kp4 + (size_t)slot * fl_warp_floats(K, M);
     float2 *LT = reinterpret_cast<float2 *>(base);  // level j: (1/T_j, P_j)
+    float *sIT = base, *sSave = base + M;           // in its place before: 1/T [M], saved flux sums [M]
     float *phi = base + 3 * M;                      // phi[-M..-1] = 0
+    float *phu = base + 5 * M;                      // phu[x] = phi[x - 1], zero below
     int *kb = (int *)(phi + M);
     float *x = (float *)(kb + M), *Sh = x + fl_k4(K), *Sf = Sh + fl_k4(K) + 4;
     float *Lw = base + fl_lw_offset(K, M);
@@ -278,32 +320,33 @@ __global__ void __launch_bounds__(fl_threads(M), fl_min_ctas(M)) k_fluct(const D
             for (int m = lo; m <= hi; ++m) kb[m] = k + 1;
         }
         __syncwarp(hmask);
+        const Pow2 nsig = pow2_pair(-sigma);  // |sigma| <= 149
         for (int m = hl; m < M; m += LW) {
             float v = 0.f;
             if (m > 0) {
                 const int a = kb[m], b = kb[m - 1];
-                v = ldexpf(Sh[a] + (Sf[b] - Sf[a]), -sigma);
+                v = (Sh[a] + (Sf[b] - Sf[a])) * nsig.a * nsig.b;
             }
             phi[m] = v;
         }
         // 4. levels owned by this lane: 1/T and the cooling factor,
         //    P_f = acc_f mul_f 2^ei_f in the frame of acc; mulx = mul 2^ei
         //    where that is a normal float (NaN otherwise: exact path)
-        float acc[MR], mul[MR], mulx[MR];
+        float acc[MR], mul[MR], mulx[MR], it[MR];
         int ei[MR];
 #pragma unroll
         for (int r = 0; r < MR; ++r) {
-            const int f = hl + LW * r;
+            const int f = level_of(r);
             acc[r] = 0.f;
             mul[r] = 0.f;
             mulx[r] = 0.f;
             ei[r] = 0;
             if (f == 0) {
-                LT[0].x = PAD_INV_T;  // level 0 (T = 0) emits nothing: every t is 0
+                it[r] = PAD_INV_T;  // level 0 (T = 0) emits nothing: every t is 0
                 continue;
             }
             const float T = gr.theta * rcp_approx(log1pf(cidE * rcp_approx((float)f)));
-            LT[f].x = rcp_approx(T);
+            it[r] = rcp_approx(T);
             // log2 of T clamped into the table: exponent split off exactly,
             // lg2.approx of the mantissa in [1/2, 1)
             const int tbits = __float_as_int(fminf(fmaxf(T, tb.Tmin), tb.Tmax));
@@ -329,6 +372,13 @@ __global__ void __launch_bounds__(fl_threads(M), fl_min_ctas(M)) k_fluct(const D
                     : ei[r] < 0 ? ldexpf(mul[r], ei[r]) : __int_as_float(0x7fc00000);
         }
         __syncwarp(hmask);
+        // phi moved up by one, over the arrays it was formed from
+        for (int m = hl; m < M; m += LW) {
+            phu[m - M] = 0.f;
+            phu[m] = phi[m - 1];
+        }
+        store_runs<RN, NR>(sIT, hl, LW, it);
+        __syncwarp(hmask);
         // 5. forward cut-flux recursion from P_0 = 1: step j adds P_j's flux
         //    to every level above j, then reads P_{j+1} off its owner lane.
         //    Level 0 sits in lane 0's first register as acc = 1 with factor 1
@@ -336,86 +386,141 @@ __global__ void __launch_bounds__(fl_threads(M), fl_min_ctas(M)) k_fluct(const D
         //    acc mul 2^ei in the current frame and a frame change rescales
         //    them all at once; the distribution is read off the registers
         //    at the end.
+        //    A lane owns runs of RN consecutive levels (one run of each RN LW
+        //    levels), so the RN values of phi that a run needs at a step are
+        //    those of the step before moved by one: RN steps read a window of
+        //    2 RN values, RN of them new.  The FMAs take levels in pairs; a
+        //    pair of phi starts at an even place on even steps and is taken
+        //    from phi, and at an odd one on odd steps and is taken from phu,
+        //    where it is even again.  Runs above the one that holds the new
+        //    levels take RN steps at once, when their P are known; runs below
+        //    it are done.  (With lanes owning every 32nd level each step
+        //    loaded each of its values: 8 instructions a step at M = 128 where
+        //    this takes 5, in four unrolled copies of the loop.)
         if (hl == 0) { acc[0] = 1.f; mul[0] = 1.f; mulx[0] = 1.f; ei[0] = 0; }
         float pj = 1.f;
-        const float *ph = phi + hl;
-        // (registers below R0 hold levels at or below j: their updates add 0)
-#define FL_STEP(J, RS, R0, OWN)                                                               \
-    {                                                                                         \
-        const int j_ = (J);                                                                   \
-        _Pragma("unroll") for (int r = (R0); r < MR; ++r) acc[r] = fmaf(ph[LW * r - j_], pj, acc[r]); \
-        const float v = __shfl_sync(hmask, acc[RS] * mulx[RS], (OWN), LW);                     \
-        if (v < 0x1p64f) {                                                                    \
-            pj = v;                                                                           \
-        } else { /* exact path: rescale the frame, or an exponent out of float range */       \
-            const float raw = __shfl_sync(hmask, acc[RS] * mul[RS], (OWN), LW);               \
-            const int E = __shfl_sync(hmask, ei[RS], (OWN), LW);                              \
-            const int ve = (raw > 0.f && raw < INFINITY) ? ilogbf(raw) : -1000;               \
-            if (ve + E > 64) {                                                                \
-                const int sh = ve + E;                                                        \
-                _Pragma("unroll") for (int r = 0; r < MR; ++r) acc[r] = ldexpf(acc[r], -sh);  \
-                pj = ldexpf(raw, -ve);                                                        \
-            } else {                                                                          \
-                pj = ldexpf(raw, E);                                                          \
-            }                                                                                 \
-        }                                                                                     \
-    }
-        // Fast form of a step: no test (a branch per step measured 12 % of
+        // acc += phi[x0 - s ...] p for the run at a, from the windows [lo | hi) of phi (s even) or phu (s odd)
+        auto add_step = [&](int s, float p, float *a, const float (&wl)[RN], const float (&wh)[RN]) {
+            const float2 p2 = make_float2(p, p);
+#pragma unroll
+            for (int r = 0; r < RN; r += 2) {
+                const int x = RN - s + r + (s & 1);  // place in the window, even
+                const float2 w = x >= RN ? make_float2(wh[x % RN], wh[x % RN + 1]) : make_float2(wl[x % RN], wl[x % RN + 1]);
+                const float2 v = __ffma2_rn(w, p2, make_float2(a[r], a[r + 1]));
+                a[r] = v.x;
+                a[r + 1] = v.y;
+            }
+        };
+        // A step has no test of its own (a branch per step measured 12 % of
         // the kernel, a flag per step 1.4 %).  A block of LW steps is checked
         // once, at its end: a block with a value past 2^100, or a level whose
         // factor is not a normal float, is taken again from its saved state
-        // with the tested step.  The check reads the block's new levels back
-        // off the registers that hold them: once its level is read, a
-        // register only takes zero terms (the pad below phi[1]), so it still
-        // gives the value that was broadcast, or NaN where a later value
-        // overflowed.  Every P of a block that passes is below 2^100, so no
-        // register can pass 2^109 (at most M <= 512 terms P phi with
-        // phi <= 1), and after each block the frame is moved to the newest
-        // level when that is above 2^32.
-#define FL_FAST(J, RS, R0, OWN)                                                               \
-    {                                                                                         \
-        const int j_ = (J);                                                                   \
-        _Pragma("unroll") for (int r = (R0); r < MR; ++r) acc[r] = fmaf(ph[LW * r - j_], pj, acc[r]); \
-        pj = __shfl_sync(hmask, acc[RS] * mulx[RS], (OWN), LW);                                \
-    }
+        // step by step.  The check reads the block's new levels back off the
+        // registers that hold them: once its level is read, a register only
+        // takes zero terms (the pad below phi[1]), so it still gives the value
+        // that was broadcast, or NaN where a later value overflowed.  Every P
+        // of a block that passes is below 2^100, so no register can pass
+        // 2^109 (at most M <= 512 terms P phi with phi <= 1), and after each
+        // block the frame is moved to the newest level when that is above 2^32.
 #pragma unroll
-        for (int r0 = 0; r0 < MR; ++r0) {
-            // block: levels LW r0 + 1 .. LW r0 + LW - 1 (this register of
-            // lanes 1..LW-1), then level LW (r0 + 1) (the next register of
-            // lane 0).  Saved state: the registers in the lanes' own LT[.].y
-            // (free until the distribution is written), and pj.
+        for (int B = 0; B < NR; ++B) {  // the run that holds the new levels: registers RN B ..
+            float we[2][RN], wo[2][RN];  // its windows of phi and phu
+            load_run<RN>(phi + RN * hl, we[1]);
+            load_run<RN>(phu + RN * hl, wo[1]);
+            // RN steps from j = RN (LW B + i); the windows' upper halves are in w[U]
+            auto steps = [&](int i, auto upper) {
+                constexpr int U = decltype(upper)::value;
+                const float *pe = phi + RN * (hl - i), *po = phu + RN * (hl - i);
+                load_run<RN>(pe - RN, we[1 - U]);
+                load_run<RN>(po - RN, wo[1 - U]);
+                float ps[RN];
 #pragma unroll
-            for (int r = 0; r < MR; ++r) LT[hl + LW * r].y = acc[r];
-            const float pj0 = pj;
-#pragma unroll 2
-            for (int jj = 0; jj < LW - 1; ++jj) FL_FAST(LW * r0 + jj, r0, r0, jj + 1)
-            if (r0 + 1 < MR) FL_FAST(LW * r0 + LW - 1, r0 + 1 < MR ? r0 + 1 : r0, r0 + 1, 0)
-            // the block's levels: register r0 of lanes 1..LW-1, and register
-            // r0 + 1 of lane 0 (read at the block's last step; none in the
-            // last block)
-            const int rb = hl > 0 ? r0 : r0 + 1;
-            float vb = 0.f;
+                for (int s = 0; s < RN; ++s) {
+                    ps[s] = pj;
+                    if (s & 1) add_step(s, pj, acc + RN * B, wo[1 - U], wo[U]);
+                    else add_step(s, pj, acc + RN * B, we[1 - U], we[U]);
+                    if (s + 1 < RN) pj = __shfl_sync(hmask, acc[RN * B + s + 1] * mulx[RN * B + s + 1], i, LW);
+                }
 #pragma unroll
-            for (int r = 0; r < MR; ++r) vb = r == rb ? acc[r] * mulx[r] : vb;
-            const bool ok = __all_sync(hmask, vb < 0x1p100f);
-            if (!ok) {  // the same on every lane of the problem (a vote)
+                for (int g = B + 1; g < NR; ++g) {
+                    const int o = (g - B) * RN * LW;
+                    float el[RN], eh[RN], ol[RN], oh[RN];
+                    load_run<RN>(pe + o - RN, el);
+                    load_run<RN>(pe + o, eh);
+                    load_run<RN>(po + o - RN, ol);
+                    load_run<RN>(po + o, oh);
 #pragma unroll
-                for (int r = 0; r < MR; ++r) acc[r] = LT[hl + LW * r].y;
+                    for (int s = 0; s < RN; ++s) {
+                        if (s & 1) add_step(s, ps[s], acc + RN * g, ol, oh);
+                        else add_step(s, ps[s], acc + RN * g, el, eh);
+                    }
+                }
+                // the next run of RN steps starts at lane i + 1's first level, or at lane 0's of the next run
+                if (i + 1 < LW) pj = __shfl_sync(hmask, acc[RN * B] * mulx[RN * B], i + 1, LW);
+                else if (B + 1 < NR) pj = __shfl_sync(hmask, acc[RN * B + RN] * mulx[RN * B + RN], 0, LW);
+            };
+#pragma unroll 1
+            for (int i0 = 0; i0 < LW; i0 += LW / RN) {
+                const int j0 = RN * (LW * B + i0);  // the block's levels: j0 + 1 .. j0 + LW
+                store_runs<RN, NR>(sSave, hl, LW, acc);
+                const float pj0 = pj;
+#pragma unroll RN == 2 ? 4 : 2
+                for (int i = i0; i < i0 + LW / RN; i += 2) {
+                    steps(i, std::integral_constant<int, 1>());
+                    steps(i + 1, std::integral_constant<int, 0>());
+                }
+                bool fine = true;
+#pragma unroll
+                for (int r = RN * B; r < MR && r <= RN * B + RN; ++r) {
+                    const int f = level_of(r);
+                    fine = fine && (f <= j0 || f > j0 + LW || acc[r] * mulx[r] < 0x1p100f);
+                }
+                if (__all_sync(hmask, fine)) {  // the same on every lane of the problem (a vote)
+                    const int e = ((__float_as_int(pj) >> 23) & 0xff) - 127;  // pj normal, < 2^100
+                    if (e > 32) {
+                        const float sc = __int_as_float((127 - e) << 23);
+#pragma unroll
+                        for (int r = 0; r < MR; ++r) acc[r] *= sc;
+                        pj *= sc;
+                    }
+                    continue;
+                }
+                load_runs<RN, NR>(sSave, hl, LW, acc);
                 pj = pj0;
-                for (int jj = 0; jj < LW - 1; ++jj) FL_STEP(LW * r0 + jj, r0, r0, jj + 1)
-                if (r0 + 1 < MR) FL_STEP(LW * r0 + LW - 1, r0 + 1 < MR ? r0 + 1 : r0, r0 + 1, 0)
-            } else {
-                const int e = ((__float_as_int(pj) >> 23) & 0xff) - 127;  // pj normal, < 2^100
-                if (e > 32) {
-                    const float sc = __int_as_float((127 - e) << 23);
+#pragma unroll 1
+                for (int i = i0; i < i0 + LW / RN; ++i) {
 #pragma unroll
-                    for (int r = 0; r < MR; ++r) acc[r] *= sc;
-                    pj *= sc;
+                    for (int st = 0; st < RN; ++st) {
+                        // the new level j + 1: register n of lane own
+                        const int j = RN * (LW * B + i) + st;
+                        const bool next = st + 1 == RN, wrap = next && i + 1 == LW;
+                        if (wrap && B + 1 == NR) break;
+                        const int own = wrap ? 0 : next ? i + 1 : i;
+#pragma unroll
+                        for (int r = RN * B; r < MR; ++r) acc[r] = fmaf(phi[level_of(r) - j], pj, acc[r]);
+                        const int n0 = RN * B + (st + 1) % RN, n1 = RN * B + RN < MR ? RN * B + RN : n0;
+                        const float A = wrap ? acc[n1] : acc[n0];
+                        const float v = __shfl_sync(hmask, A * (wrap ? mulx[n1] : mulx[n0]), own, LW);
+                        if (v < 0x1p64f) {
+                            pj = v;
+                            continue;
+                        }
+                        // rescale the frame, or an exponent out of float range
+                        const float raw = __shfl_sync(hmask, A * (wrap ? mul[n1] : mul[n0]), own, LW);
+                        const int E = __shfl_sync(hmask, wrap ? ei[n1] : ei[n0], own, LW);
+                        const int ve = (raw > 0.f && raw < INFINITY) ? ilogbf(raw) : -1000;
+                        if (ve + E > 64) {
+                            const int sh = ve + E;
+#pragma unroll
+                            for (int r = 0; r < MR; ++r) acc[r] = ldexpf(acc[r], -sh);
+                            pj = ldexpf(raw, -ve);
+                        } else {
+                            pj = ldexpf(raw, E);
+                        }
+                    }
                 }
             }
         }
-#undef FL_FAST
-#undef FL_STEP
         // the distribution in the final frame, normalised
         float pv[MR], z = 0.f;
 #pragma unroll
@@ -427,12 +532,21 @@ __global__ void __launch_bounds__(fl_threads(M), fl_min_ctas(M)) k_fluct(const D
 #pragma unroll
         for (int o = LW / 2; o; o >>= 1) z += __shfl_xor_sync(hmask, z, o);
         const float iz = 1.f / z;
+        load_runs<RN, NR>(sIT, hl, LW, it);
+        __syncwarp(hmask);  // LT overwrites sIT and sSave
 #pragma unroll
-        for (int r = 0; r < MR; ++r) {
-            const int j = hl + LW * r;
-            const float p = pv[r] * iz;
-            LT[j].y = p;
-            if (P) P[((size_t)c * fd.Gf + q) * M + j] = p;
+        for (int r = 0; r < MR; ++r) pv[r] *= iz;
+#pragma unroll
+        for (int r = 0; r < MR; r += 2)
+            *reinterpret_cast<float4 *>(LT + level_of(r)) = make_float4(it[r], pv[r], it[r + 1], pv[r + 1]);
+        if (P) {
+            float *row = P + ((size_t)c * fd.Gf + q) * M;
+            if ((reinterpret_cast<uintptr_t>(P) & 15) == 0) {
+                store_runs<RN, NR>(row, hl, LW, pv);
+            } else {
+#pragma unroll
+                for (int r = 0; r < MR; ++r) row[level_of(r)] = pv[r];
+            }
         }
         if (dE_out && hl == 0) dE_out[c * fd.Gf + q] = dEt * eps_ref;
         __syncwarp(hmask);
