@@ -4,11 +4,14 @@ Argument marshalling only: every step of the path runs in the library's CUDA
 kernels.  Loading fails loudly when libdust.so has not been built.
 """
 import ctypes
+import importlib.util
 import os
 import re
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(HERE, "_build", "libdust.so")
+FRONT_PATH = os.path.join(HERE, "_build", "_front" + sysconfig.get_config_var("EXT_SUFFIX"))
 HEADER = os.path.join(os.path.dirname(HERE), "include", "dust.h")
 
 DUST_OK, DUST_EINVAL, DUST_ENOMEM, DUST_ECUDA, DUST_EBUSY, DUST_ETIMEOUT, DUST_ENOTFOUND = range(7)
@@ -90,6 +93,30 @@ def lib():
             fn.argtypes = args
         _lib = L
     return _lib
+
+
+_front = None
+
+
+def front():
+    """The front end's native half, csrc/front.cpp (raises if it has not been built)."""
+    global _front
+    if _front is None:
+        if not os.path.exists(FRONT_PATH):
+            raise RuntimeError(f"the front end is not built ({FRONT_PATH} missing): run "
+                               "`python -c 'import __graft_entry__ as g; g.build()'`")
+        import torch  # noqa: F401  (its libraries have to be loaded first)
+
+        spec = importlib.util.spec_from_file_location("_front", FRONT_PATH)
+        m = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(m)
+        _front = m
+    return _front
+
+
+def address(name):
+    """Address of a function of the library."""
+    return ctypes.cast(getattr(lib(), name), _p).value
 
 
 def last_error():

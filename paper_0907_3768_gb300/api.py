@@ -51,6 +51,8 @@ class Context:
                                            int(device))
         self.K, self.G, self.device = K, G, int(device)
         self.T_min, self.T_max = float(T_min), float(T_max)
+        self._front = _lib.front()
+        self._solve, self._solve_mass = _lib.address("dust_solve"), _lib.address("dust_solve_mass")
 
     @classmethod
     def from_workload(cls, wl, precision="fp32", device=0):
@@ -109,18 +111,27 @@ class Context:
         return C, J.stride(0)
 
     def alloc_outputs(self, C, ld, want_L=True, want_resid=True, want_flags=True):
-        dev = torch.device("cuda", self.device)
-        out = dict(T=torch.empty((C, self.G), dtype=torch.float32, device=dev))
-        out["L_buf"] = torch.empty((C, ld), dtype=torch.float32, device=dev) if want_L else None
-        out["L"] = out["L_buf"][:, :self.K] if want_L else None
-        out["resid"] = torch.empty((C,), dtype=torch.float64, device=dev) if want_resid else None
-        out["flags"] = torch.empty((C, self.G), dtype=torch.uint8, device=dev) if want_flags else None
-        return out
+        return self._front.alloc_outputs(C, self.G, self.K, ld, self.device, want_L, want_resid, want_flags)
+
+    def _solve_new(self, fn, J, n, mass, want_L, want_resid, want_flags):
+        """One native call into new outputs on the current stream; None where J or n is not what it takes."""
+        if self.handle is None or not isinstance(J, torch.Tensor) or not isinstance(n, torch.Tensor):
+            return None
+        r = self._front.solve(fn, self.handle, self.G, self.K, self.device, J, n, mass, bool(want_L), bool(want_resid),
+                              bool(want_flags))
+        if r is None:
+            return None
+        _lib.check(r[1])
+        return r[0]
 
     def solve(self, J, n, precision=None, want_L=True, want_resid=True, want_flags=True, out=None,
               stream=None):
         """Run the hot path on device tensors; returns a dict of output tensors
         (T [C,G], L [C,K] view, resid [C] float64, flags [C,G] uint8)."""
+        if out is None and stream is None and precision is None:
+            new = self._solve_new(self._solve, J, n, False, want_L, want_resid, want_flags)
+            if new is not None:
+                return new
         C, ld = self._check_inputs(J, n)
         if out is None:
             out = self.alloc_outputs(C, ld, want_L, want_resid, want_flags)
@@ -162,6 +173,10 @@ class Context:
     def solve_mass(self, J, m, out=None, want_L=True, want_resid=True, want_flags=True, stream=None):
         """The hot path with n[c,g] = n_g m_c (Eqs. 9-10): m [C] float32 CUDA
         tensor of the cells' dust masses; outputs as solve()."""
+        if out is None and stream is None:
+            new = self._solve_new(self._solve_mass, J, m, True, want_L, want_resid, want_flags)
+            if new is not None:
+                return new
         C = J.shape[0]
         if m.shape != (C,) or m.dtype != torch.float32 or not m.is_cuda or not m.is_contiguous():
             raise ValueError("m must be a contiguous float32 CUDA tensor of shape [C]")

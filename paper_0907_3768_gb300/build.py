@@ -1,4 +1,5 @@
-"""In-tree build of libdust.so for sm_103a (nvcc, no cmake).
+"""In-tree build of libdust.so for sm_103a (nvcc, no cmake) and of _front, the
+front end's native half (g++, against the installed torch's headers).
 
 Each .cu under csrc/ is compiled to an object in parallel, then linked into
 paper_0907_3768_gb300/_build/libdust.so with the CUDA runtime linked
@@ -10,11 +11,14 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libdust.so")
+FRONT_SRC = os.path.join(CSRC, "front.cpp")
+FRONT = os.path.join(OUT, "_front" + sysconfig.get_config_var("EXT_SUFFIX"))
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
@@ -44,7 +48,38 @@ def up_to_date():
     return all(os.path.getmtime(p) <= t for p in _deps())
 
 
+def build_front(force=False):
+    """Compile and link the _front module; returns its path."""
+    deps = [FRONT_SRC, os.path.join(INCLUDE, "dust.h")]
+    if not force and os.path.exists(FRONT) and all(os.path.getmtime(p) <= os.path.getmtime(FRONT) for p in deps):
+        return FRONT
+    import torch
+    from torch.utils import cpp_extension
+
+    os.makedirs(OUT, exist_ok=True)
+    inc = [*cpp_extension.include_paths("cuda"), "/usr/local/cuda/include", sysconfig.get_path("include")]
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    tmp = FRONT + f".tmp{os.getpid()}"
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           *["-I" + p for p in inc], FRONT_SRC, "-o", tmp, "-L" + lib, "-Wl,-rpath," + lib,
+           "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch", "-ltorch_python"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed on front.cpp:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, FRONT)
+    return FRONT
+
+
 def build(force=False, verbose=False, ptxas_verbose=False):
+    """Compile and link libdust.so and the _front module; returns libdust.so's path."""
+    with cf.ThreadPoolExecutor(max_workers=1) as ex:
+        front = ex.submit(build_front, force)
+        lib = build_lib(force, verbose, ptxas_verbose)
+        front.result()
+    return lib
+
+
+def build_lib(force=False, verbose=False, ptxas_verbose=False):
     """Compile and link libdust.so; returns its path."""
     if not force and up_to_date():
         return LIB
