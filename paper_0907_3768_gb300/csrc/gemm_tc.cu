@@ -48,14 +48,13 @@ constexpr int FUSED_NS1 = 2, FUSED_NS2 = 2;          // fused kernel: ring depth
 constexpr int STAGE1_BYTES = BM * KC * 4;  // FP32 staging tile: 16 KB
 constexpr int A_BYTES = BM * KC * 2;       // one 16-bit A part: 8 KB
 // grain-major orientation (Gs <= 128): grains are the MMA's M, cells its N
-constexpr int BN_T = 256;                     // cells per tile (UMMA N)
+constexpr int BN_T = 256, BN_S = 64;          // cells per tile (UMMA N): long and short tiles
 constexpr int MW = 128;                       // grain rows of the W operand (UMMA M; zero past Gs)
-constexpr int STAGE1T_BYTES = BN_T * KC * 4;  // FP32 staging tile: 32 KB
 constexpr int WA_PART = MW * KC * 2;          // one 16-bit W part: 8 KB
-constexpr int JB_PART = BN_T * KC * 2;        // one 16-bit J part: 16 KB
-constexpr int TN_NS1 = 4, TN_NS2 = 2;         // its ring depths, at most
+__host__ __device__ constexpr int stage1t_bytes(int bn) { return bn * KC * 4; }  // FP32 staging tile: 32 KB at 256 cells
+__host__ __device__ constexpr int jb_part(int bn) { return bn * KC * 2; }        // one 16-bit J part: 16 KB at 256
+constexpr int TN_NS1 = 4, TN_NS2 = 2;         // its ring depths at 256 cells, at most
 constexpr int NCV_T = 8;                      // its converter warps
-constexpr int RPT = BN_T / (32 * NCV_T);      // cell rows per converter thread
 constexpr int NTHREADS_T = (3 + NCV_T + 4) * 32;
 
 // ---------------------------------------------------------------- PTX helpers
@@ -599,20 +598,32 @@ __global__ void __launch_bounds__(NTHREADS_F, 1) k_absorb_solve(const __grid_con
 }
 
 // Grain-major form of the same contraction for Gs <= 128: W (grains x K,
-// zero rows up to 128) is the MMA's A operand and a 256-cell tile of J its B
-// operand, so one MMA covers twice the cells of the cell-major kernel at
-// about the same issue cost; the accumulator is 128 grain lanes x 256 cell
-// columns.  Roles as in k_gemm_tc: warp 0 J producer (TMA, 256-row boxes),
-// warp 1 tensor memory + MMA issuer, warp 2 W producer (two bulk copies per
-// chunk: hi and lo parts into their 128-row slots), then NCV_T converter
-// warps (256 / (32 NCV_T) cell rows per thread) and four epilogue warps
-// (thread = grain, 32 cell columns per tensor-memory load; each store of a
-// warp is 32 consecutive grains of one cell row of S).
-template <bool BF16, bool TWO_PASS>
+// zero rows up to 128) is the MMA's A operand and a tile of bn cells of J
+// (256, or 64 in small calls) its B operand, so one MMA covers twice the
+// cells of the cell-major kernel at about the same issue cost; the
+// accumulator is 128 grain lanes x bn cell columns.  Roles as in k_gemm_tc:
+// warp 0 J producer (TMA, bn-row boxes), warp 1 tensor memory + MMA issuer,
+// warp 2 W producer (two bulk copies per chunk: hi and lo parts into their
+// 128-row slots), then NCV_T converter warps (one cell row per thread, or a
+// half or a quarter of one in short tiles) and four epilogue warps (thread =
+// grain, 32 cell columns per tensor-memory load; each store of a warp is 32
+// consecutive grains of one cell row of S).
+// Short tiles (bn = 64, up to as many as there are SMs): with 256 a call of 32
+// cells converted and multiplied 224 empty rows, 12.5 us against 9.3; tiles of
+// just the cells per SM, with bn read at run time, were slower at every other
+// size (20011 cells 13.8 us in 139 tiles of 144, 12.7 in 79 of 256; 262144
+// cells 74 us against 56), since the addresses of each role's loop pace it.
+// FP16 reads a tile twice (its cells' exponents, then the conversion); it was
+// bound by its epilogue, which built two powers of two per value from the
+// exponents: the converters leave them in shared memory (262144 x 200 x 96: 95
+// -> 80 us).  A ring that holds the tile for the second reading was slower (89
+// us: two stages are left for the next tile).
+template <bool BF16, bool TWO_PASS, int BN>
 __global__ void __launch_bounds__(NTHREADS_T, 1) k_gemm_tc_t(const __grid_constant__ TcBatch p) {
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
     unsigned char *st1 = smem;                                        // [ns1] FP32 J tiles
+    constexpr int bn = BN, STAGE1T_BYTES = stage1t_bytes(bn), JB_PART = jb_part(bn);
     unsigned char *stW = st1 + (size_t)p.ns1 * STAGE1T_BYTES;         // [ns2] W hi | lo
     unsigned char *stJ = stW + (size_t)p.ns2 * 2 * WA_PART;           // [ns2] J hi | lo
     uint64_t *bars = (uint64_t *)(stJ + (size_t)p.ns2 * 2 * JB_PART);
@@ -620,7 +631,7 @@ __global__ void __launch_bounds__(NTHREADS_T, 1) k_gemm_tc_t(const __grid_consta
     uint64_t *w_full = empty1 + p.ns1, *j_full = w_full + p.ns2, *ab_empty = j_full + p.ns2;
     uint64_t *acc_full = ab_empty + p.ns2, *acc_empty = acc_full + 2;
     uint64_t *e_full = acc_empty + 2, *e_empty = e_full + 2, *drain = e_empty + 2;
-    int *e_smem = (int *)(drain + 1);                 // [2][BN_T] per-cell exponents
+    Pow2 *e_smem = (Pow2 *)(drain + 1);               // [2][BN_T] per-cell scales back, 2^(e - j_off - off_exp)
     uint32_t *tmem_slot = (uint32_t *)(e_smem + 2 * BN_T);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
 
@@ -668,7 +679,7 @@ __global__ void __launch_bounds__(NTHREADS_T, 1) k_gemm_tc_t(const __grid_consta
                 ri = tc_req_of(p, tile, ri);
                 const TcReq &q = p.req[ri];
                 const CUtensorMap *tm = &p.tm[ri];
-                const int row0 = (int)((tile - q.tile_begin) * BN_T);
+                const int row0 = (int)((tile - q.tile_begin) * bn);
                 for (int pass = TWO_PASS ? 0 : 1; pass < 2 && ok; ++pass) {
                     for (int kc = 0; kc < q.nkc && ok; ++kc) {
                         if (!(ok = mbar_wait(&empty1[s1], ph1 ^ 1, abort_flag, p.status))) break;
@@ -712,7 +723,13 @@ __global__ void __launch_bounds__(NTHREADS_T, 1) k_gemm_tc_t(const __grid_consta
             uint32_t pha = 0;
             int64_t it = 0;
             bool ok = true;
-            const uint32_t idesc = instr_desc(BF16, MW, BN_T);
+            const uint32_t idesc = instr_desc(BF16, MW, bn);
+            // operand descriptors of slot 0, part hi, K step 0; a slot, a part and
+            // a K step away are sums in their address field (16-byte units, no
+            // carry out of it below 256 KB): this thread's own instructions pace
+            // the MMAs
+            const uint64_t wd0 = smem_desc(smem_u32(stW), 128, 512), jd0 = smem_desc(smem_u32(stJ), 128, 512);
+            const uint64_t w_slot = 2 * WA_PART / 16, j_slot = 2 * JB_PART / 16, w_lo = WA_PART / 16, j_lo = JB_PART / 16;
             for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++it) {
                 ri = tc_req_of(p, tile, ri);
                 const int nkc = p.req[ri].nkc, np = p.req[ri].nparts;
@@ -722,23 +739,16 @@ __global__ void __launch_bounds__(NTHREADS_T, 1) k_gemm_tc_t(const __grid_consta
                 if (!(ok = mbar_wait(&acc_empty[b], ub ^ 1, abort_flag, p.status))) break;
                 tc_fence_after();
                 for (int kc = 0; kc < nkc && ok; ++kc) {
+                    const uint64_t wd = wd0 + sa * w_slot, jd = jd0 + sa * j_slot;
                     if (!(ok = mbar_wait(&w_full[sa], pha, abort_flag, p.status))) break;
                     if (!(ok = mbar_wait(&j_full[sa], pha, abort_flag, p.status))) break;
                     tc_fence_after();
-                    const uint32_t w_base = smem_u32(stW + (size_t)sa * 2 * WA_PART);
-                    const uint32_t j_base = smem_u32(stJ + (size_t)sa * 2 * JB_PART);
 #pragma unroll
                     for (int ks = 0; ks < KC / 16; ++ks) {
-#pragma unroll
-                        for (int part = 0; part < 3; ++part) {
-                            // W hi . J hi, W hi . J lo, W lo . J hi (np = 2: the last left out)
-                            if (part >= np) break;
-                            const uint32_t woff = (part == 2 ? WA_PART : 0) + ks * 256;
-                            const uint32_t joff = (part == 1 ? JB_PART : 0) + ks * 256;
-                            const uint32_t acc = (kc | ks | part) ? 1u : 0u;
-                            tc_mma(d_tmem, smem_desc(w_base + woff, 128, 512), smem_desc(j_base + joff, 128, 512),
-                                   idesc, acc);
-                        }
+                        // W hi . J hi, W hi . J lo, W lo . J hi (np = 2: the last left out)
+                        tc_mma(d_tmem, wd + 16 * ks, jd + 16 * ks, idesc, (kc | ks) ? 1u : 0u);
+                        tc_mma(d_tmem, wd + 16 * ks, jd + 16 * ks + j_lo, idesc, 1u);
+                        if (np > 2) tc_mma(d_tmem, wd + 16 * ks + w_lo, jd + 16 * ks, idesc, 1u);
                     }
                     tc_commit(&ab_empty[sa]);
                     if (++sa == p.ns2) { sa = 0; pha ^= 1; }
@@ -751,7 +761,13 @@ __global__ void __launch_bounds__(NTHREADS_T, 1) k_gemm_tc_t(const __grid_consta
         }
     } else if (warp < 3 + NCV_T) {
         // ------------------------------------------------------------ converters
-        const int r0 = (warp - 3) * 32 + lane;  // cell rows r0 + h NCV_T 32 of the tile, h < RPT
+        // cell row r of the tile, core-matrix columns [cm0, cm1) of its four: a whole
+        // row per thread, or a half or a quarter where the tile has no more
+        // rows than half or a quarter of the threads
+        const int ct = (warp - 3) * 32 + lane;
+        const int rows = bn > 128 ? 256 : bn > 64 ? 128 : 64, per = 4 * rows / 256;
+        const int r = ct % rows, cm0 = ct / rows * per, cm1 = cm0 + per;
+        const bool on = r < bn;
         int s1 = 0, sa = 0, ri = 0;
         uint32_t ph1 = 0, pha = 0;
         int64_t it = 0;
@@ -759,19 +775,17 @@ __global__ void __launch_bounds__(NTHREADS_T, 1) k_gemm_tc_t(const __grid_consta
         for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++it) {
             ri = tc_req_of(p, tile, ri);
             const TcReq &q = p.req[ri];
-            int e[RPT] = {};
+            int e = 0;
             if (TWO_PASS) {
-                float mx[RPT] = {};
+                float mx = 0.f;
                 for (int kc = 0; kc < q.nkc; ++kc) {
                     if (!(ok = mbar_wait(&full1[s1], ph1, abort_flag, p.status))) break;
-#pragma unroll
-                    for (int h = 0; h < RPT; ++h) {
-                        const int r = r0 + h * NCV_T * 32;
+                    if (on) {
                         const unsigned char *src = st1 + (size_t)s1 * STAGE1T_BYTES + r * 128;
 #pragma unroll
                         for (int j = 0; j < 8; ++j) {
                             float4 v = *reinterpret_cast<const float4 *>(src + ((j ^ (r & 7)) << 4));
-                            mx[h] = fmaxf(mx[h], fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+                            mx = fmaxf(mx, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
                         }
                     }
                     __syncwarp();
@@ -779,43 +793,40 @@ __global__ void __launch_bounds__(NTHREADS_T, 1) k_gemm_tc_t(const __grid_consta
                     if (++s1 == p.ns1) { s1 = 0; ph1 ^= 1; }
                 }
                 if (!ok) break;
-#pragma unroll
-                for (int h = 0; h < RPT; ++h) {
-                    if (mx[h] > 0.f && mx[h] < INFINITY) frexpf(mx[h], &e[h]);
-                    e[h] = min(max(e[h], p.j_off - 126), p.j_off + 126);  // keep 2^(j_off - e) a normal float
-                }
-                // hand the exponents to the epilogue
+                if (mx > 0.f && mx < INFINITY) frexpf(mx, &e);
+                e = min(max(e, p.j_off - 126), p.j_off + 126);  // keep 2^(j_off - e) a normal float
+                // hand the scales to the epilogue
                 const int b = (int)(it & 1);
                 const uint32_t ub = (uint32_t)((it >> 1) & 1);
                 if (!(ok = mbar_wait(&e_empty[b], ub ^ 1, abort_flag, p.status))) break;
-#pragma unroll
-                for (int h = 0; h < RPT; ++h) e_smem[b * BN_T + r0 + h * NCV_T * 32] = e[h];
+                if (on && cm0 == 0) e_smem[b * BN_T + r] = pow2_pair(e - p.j_off - p.off_exp);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&e_full[b]);
             }
-            float scale[RPT];
-#pragma unroll
-            for (int h = 0; h < RPT; ++h) scale[h] = __int_as_float((127 - e[h] + p.j_off) << 23);  // 2^(j_off - e)
+            const float scale = __int_as_float((127 - e + p.j_off) << 23);  // 2^(j_off - e)
             for (int kc = 0; kc < q.nkc; ++kc) {
                 if (!(ok = mbar_wait(&full1[s1], ph1, abort_flag, p.status))) break;
                 if (!(ok = mbar_wait(&ab_empty[sa], pha ^ 1, abort_flag, p.status))) break;
-#pragma unroll
-                for (int h = 0; h < RPT; ++h) {
-                    const int r = r0 + h * NCV_T * 32;
+                if (on) {
                     const unsigned char *src = st1 + (size_t)s1 * STAGE1T_BYTES + r * 128;
                     unsigned char *dhi = stJ + (size_t)sa * 2 * JB_PART + (r >> 3) * 512 + (r & 7) * 16;
                     unsigned char *dlo = dhi + JB_PART;
-#pragma unroll
-                    for (int cm = 0; cm < 4; ++cm) {  // 8 wavelengths = one core-matrix row
+                    auto convert = [&](int cm) {  // 8 wavelengths = one core-matrix row
                         float4 v0 = *reinterpret_cast<const float4 *>(src + (((2 * cm) ^ (r & 7)) << 4));
                         float4 v1 = *reinterpret_cast<const float4 *>(src + (((2 * cm + 1) ^ (r & 7)) << 4));
                         uint4 hv, lv;
-                        hv.x = pack_split(v0.x * scale[h], v0.y * scale[h], BF16, lv.x);
-                        hv.y = pack_split(v0.z * scale[h], v0.w * scale[h], BF16, lv.y);
-                        hv.z = pack_split(v1.x * scale[h], v1.y * scale[h], BF16, lv.z);
-                        hv.w = pack_split(v1.z * scale[h], v1.w * scale[h], BF16, lv.w);
+                        hv.x = pack_split(v0.x * scale, v0.y * scale, BF16, lv.x);
+                        hv.y = pack_split(v0.z * scale, v0.w * scale, BF16, lv.y);
+                        hv.z = pack_split(v1.x * scale, v1.y * scale, BF16, lv.z);
+                        hv.w = pack_split(v1.z * scale, v1.w * scale, BF16, lv.w);
                         *reinterpret_cast<uint4 *>(dhi + cm * 128) = hv;
                         *reinterpret_cast<uint4 *>(dlo + cm * 128) = lv;
+                    };
+                    if (per == 4) {
+#pragma unroll
+                        for (int cm = 0; cm < 4; ++cm) convert(cm);
+                    } else {
+                        for (int cm = cm0; cm < cm1; ++cm) convert(cm);
                     }
                 }
                 fence_proxy_async();
@@ -841,20 +852,20 @@ __global__ void __launch_bounds__(NTHREADS_T, 1) k_gemm_tc_t(const __grid_consta
             if (!(ok = mbar_wait(&acc_full[b], ub, abort_flag, p.status))) break;
             tc_fence_after();
             const int Gs = q.Gs;
-            const int64_t cell0 = (tile - q.tile_begin) * BN_T;
-            const int nc = (int)min((int64_t)BN_T, q.C - cell0);  // cells of this tile
+            const int64_t cell0 = (tile - q.tile_begin) * bn;
+            const int nc = (int)min((int64_t)bn, q.C - cell0);  // cells of this tile
             const uint32_t tbase = tmem + (uint32_t)(b * BN_T) + ((uint32_t)(quad * 32) << 16);
             if (quad * 32 < Gs) {  // warp-uniform: quarters past the grains hold zeros only
                 float *col = q.S + cell0 * Gs + g;  // S[cell0][g]
                 const bool gok = g < Gs;
-                const int ex0 = -p.j_off - p.off_exp;
-                for (int c0 = 0; c0 < BN_T; c0 += 32) {
+                const Pow2 all = pow2_pair(-p.j_off - p.off_exp);  // BF16: every cell's
+                for (int c0 = 0; c0 < BN; c0 += 32) {
                     float v[32];
                     tmem_ld32(tbase + (uint32_t)c0, v);
 #pragma unroll
                     for (int i = 0; i < 32; ++i) {
-                        const int ex = (TWO_PASS ? e_smem[b * BN_T + c0 + i] : 0) + ex0;
-                        if (gok && c0 + i < nc) col[(c0 + i) * Gs] = scale2(v[i], ex);
+                        const Pow2 f = TWO_PASS ? e_smem[b * BN_T + c0 + i] : all;
+                        if (gok && c0 + i < nc) col[(c0 + i) * Gs] = v[i] * f.a * f.b;
                     }
                 }
             }
@@ -893,7 +904,7 @@ static_assert(sizeof(TcBatch) + sizeof(SolveList) <= 32764, "fused launch parame
 template <bool BF16, bool TWO_PASS>
 int launch_t(const TcBatch &B, size_t smem, int grid, cudaStream_t st, const SolveList *sl) {
     if (B.orient == 1) {
-        auto kern = k_gemm_tc_t<BF16, TWO_PASS>;
+        auto kern = B.bn == BN_T ? k_gemm_tc_t<BF16, TWO_PASS, BN_T> : k_gemm_tc_t<BF16, TWO_PASS, BN_S>;
         DUST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         kern<<<grid, NTHREADS_T, smem, st>>>(B);
     } else if (sl) {
@@ -918,8 +929,11 @@ int launch_t(const TcBatch &B, size_t smem, int grid, cudaStream_t st, const Sol
 
 int tc_orient(const dust_ctx *ctx) { return ctx->tb.Gs <= MW ? 1 : 0; }
 
+// Short tiles while they are no more than the SMs.
+int tc_tile_cells(int64_t cells, int num_sms) { return cells <= (int64_t)BN_S * num_sms ? BN_S : BN_T; }
+
 int make_tc_req(const dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t ld, float *S, TcReq &r,
-                CUtensorMap &tm, int orient) {
+                CUtensorMap &tm, int orient, int bn) {
     const bool bf16 = precision == DUST_PREC_BF16X3;
     const int K = ctx->K;
     if (C > 0x7fffffffLL - BN_T) return set_error(DUST_EINVAL, "too many cells for one tensor-core launch");
@@ -928,7 +942,7 @@ int make_tc_req(const dust_ctx *ctx, int precision, int64_t C, const float *J, i
     cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)C};
     cuuint64_t strides[1] = {(cuuint64_t)ld * sizeof(float)};
     if (orient == 1 && ctx->tb.Gs > MW) return set_error(DUST_EINVAL, "grain-major GEMM needs Gs <= %d", MW);
-    cuuint32_t box[2] = {(cuuint32_t)KC, (cuuint32_t)(orient == 1 ? BN_T : BM)};
+    cuuint32_t box[2] = {(cuuint32_t)KC, (cuuint32_t)(orient == 1 ? bn : BM)};
     cuuint32_t estr[2] = {1, 1};
     CUresult cr = encode(&tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, (void *)J, dims, strides, box, estr,
                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -947,7 +961,7 @@ int make_tc_req(const dust_ctx *ctx, int precision, int64_t C, const float *J, i
 // Tile offsets, ring depths and tensor-memory layout of a filled batch.
 int finish_tc_batch(TcBatch &B, int precision, size_t smem_optin, size_t *smem, bool fused) {
     const bool bf16 = precision == DUST_PREC_BF16X3;
-    const int bm = B.orient == 1 ? BN_T : BM;
+    const int bm = B.orient == 1 ? B.bn : BM;
     int64_t t = 0;
     int gmax = 16;
     for (int i = 0; i < B.nreq; ++i) {
@@ -964,11 +978,12 @@ int finish_tc_batch(TcBatch &B, int precision, size_t smem_optin, size_t *smem, 
         B.nacc = 2;
         B.j_off = bf16 ? 0 : 15;
         B.off_exp = bf16 ? 0 : 14;
+        const int bn = B.bn;
         auto need_t = [&](int a, int b) {
-            return (size_t)a * STAGE1T_BYTES + (size_t)b * 2 * (WA_PART + JB_PART) + (size_t)(2 * a + 3 * b + 9) * 8 +
-                   2 * BN_T * 4 + 16;
+            return (size_t)a * stage1t_bytes(bn) + (size_t)b * 2 * (WA_PART + jb_part(bn)) + (size_t)(2 * a + 3 * b + 9) * 8 +
+                   2 * BN_T * sizeof(Pow2) + 16;
         };
-        int ns1 = TN_NS1, ns2 = TN_NS2;
+        int ns1 = bn == BN_T ? TN_NS1 : 2 * TN_NS1, ns2 = TN_NS2;
         while (need_t(ns1, ns2) > budget && ns1 > 2) --ns1;
         while (need_t(ns1, ns2) > budget && ns2 > 2) --ns2;
         if (need_t(ns1, ns2) > budget) return set_error(DUST_EINVAL, "shared memory too small for the grain-major GEMM");
@@ -1024,7 +1039,8 @@ int launch_gemm_tc(const dust_ctx *ctx, int precision, int64_t C, const float *J
     B.nzero = nzero;
     B.status = ctx->tb.status;
     B.orient = tc_orient(ctx);
-    int rc = make_tc_req(ctx, precision, C, J, ld, S, B.req[0], B.tm[0], B.orient);
+    B.bn = tc_tile_cells(C, ctx->num_sms);
+    int rc = make_tc_req(ctx, precision, C, J, ld, S, B.req[0], B.tm[0], B.orient, B.bn);
     if (rc != DUST_OK) return rc;
     size_t smem = 0;
     if ((rc = finish_tc_batch(B, precision, ctx->smem_optin, &smem)) != DUST_OK) return rc;

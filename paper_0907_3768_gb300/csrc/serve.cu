@@ -314,13 +314,17 @@ int launch_round(dust_server *s, const Round &rd) {
                 B.nzero = 0;
                 B.status = nullptr;
                 B.orient = orient;
+                int64_t cells = 0;
+                for (const Part &p : parts)
+                    if (p.r->precision == prec && tc_orient(p.r->ctx) == orient) cells += p.cn;
+                B.bn = tc_tile_cells(cells, s->num_sms);
                 for (size_t k = 0; k < parts.size(); ++k) {
                     const Part &p = parts[k];
                     if (p.r->precision != prec || tc_orient(p.r->ctx) != orient) continue;
                     ServeReq *r = p.r;
                     if (!B.status) B.status = r->ctx->tb.status;
                     int rc = make_tc_req(r->ctx, prec, p.cn, r->J + p.c0 * r->ld, r->ld, part_view(s, p, rd.slot, (int)k).S,
-                                         B.req[B.nreq], B.tm[B.nreq], orient);
+                                         B.req[B.nreq], B.tm[B.nreq], orient, B.bn);
                     if (rc != DUST_OK) return rc;
                     B.nreq++;
                 }
