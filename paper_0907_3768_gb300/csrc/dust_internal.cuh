@@ -367,14 +367,16 @@ int ensure_scratch(dust_ctx *ctx, int64_t cells, cudaStream_t st);
 // request's, or a slice of one: order, classes and counts may be NULL, and
 // the cells are then emitted in ascending order); nlaunch counts the kernels,
 // ev (optional, four events) marks absorption / solve / emission boundaries.
+// keep_order: the scratch still holds the emission order that the last call
+// made for as many cells; it is taken as it is.
 int solve_view(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t ld, const float *n, float *T,
                float *L, double *resid, uint8_t *flags, const ScratchView &sv, cudaStream_t st, bool mass,
-               int *nlaunch, cudaEvent_t *ev = nullptr);
+               int *nlaunch, cudaEvent_t *ev = nullptr, bool keep_order = false);
 // The whole path on device buffers with scratch of scratch_bytes(ctx, C, true)
 // bytes at `scratch`.
 int solve_device(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t ld,
                  const float *n, float *T, float *L, double *resid, uint8_t *flags, void *scratch,
-                 cudaStream_t st, bool mass = false);
+                 cudaStream_t st, bool mass = false, bool keep_order = false);
 
 // Bounded spin budget for device-side waits: a wait that exceeds it records
 // DUST_ETIMEOUT in the status word and gives up.

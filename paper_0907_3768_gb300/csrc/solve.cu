@@ -90,7 +90,7 @@ cudaEvent_t prof_event(dust_ctx *ctx) {
 
 int solve_view(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t ld, const float *n, float *T,
                float *L, double *resid, uint8_t *flags, const ScratchView &sv, cudaStream_t st, bool mass,
-               int *nlaunch, cudaEvent_t *ev) {
+               int *nlaunch, cudaEvent_t *ev, bool keep_order) {
     int nl_total = 0;
     if (nlaunch) *nlaunch = 0;
     if (C == 0) return DUST_OK;
@@ -133,7 +133,9 @@ int solve_view(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t 
     // 32-cell tiles; it never changes a result.  Small calls skip it: there the
     // ordering's three launches cost more than the warp-uniform regimes save.
     const bool ordered = !split.parts && C > (int64_t)32 * ctx->num_sms;
-    if (rc == DUST_OK && (L || resid) && ordered && sv.order && sv.bkt && sv.hist) {
+    if (keep_order && (L || resid) && ordered && sv.order && sv.bkt && sv.hist) {
+        B.req[0].order = sv.order;
+    } else if (rc == DUST_OK && (L || resid) && ordered && sv.order && sv.bkt && sv.hist) {
         // emission order: cells classed by the absorbed power of the reference
         // grain (S), or by its inverse temperature where S stayed in tensor memory
         const int gref = order_ref_grain(ctx->G);
@@ -185,7 +187,8 @@ int solve_view(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t 
 }
 
 int solve_device(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t ld, const float *n,
-                 float *T, float *L, double *resid, uint8_t *flags, void *scratch, cudaStream_t st, bool mass) {
+                 float *T, float *L, double *resid, uint8_t *flags, void *scratch, cudaStream_t st, bool mass,
+                 bool keep_order) {
     if (C == 0) return DUST_OK;
     const ScratchView sv = scratch_view(ctx, C, scratch);
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -193,7 +196,7 @@ int solve_device(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_
         for (int i = 0; i < 4; ++i) ev[i] = prof_event(ctx);
     const bool prof = ev[0] && ev[1] && ev[2] && ev[3];
     int nl = 0;
-    const int rc = solve_view(ctx, precision, C, J, ld, n, T, L, resid, flags, sv, st, mass, &nl, prof ? ev : nullptr);
+    const int rc = solve_view(ctx, precision, C, J, ld, n, T, L, resid, flags, sv, st, mass, &nl, prof ? ev : nullptr, keep_order);
     ctx->launches += (uint64_t)nl;
     for (int i = 0; i < 4; ++i) {
         if (!ev[i]) continue;
