@@ -135,7 +135,7 @@ struct OrderReq {
     const float *key;
     int64_t kstride, C;
     uint16_t *bkt;
-    unsigned *hist;  // [2][NBK], zeroed by the launch
+    unsigned *hist;  // [2][NBK], zeroed before classify
     int *order;
     int block_begin;  // first CTA of the request in the classify / scatter grids
 };
@@ -297,6 +297,37 @@ const char *cuda_err_name(cudaError_t e);
         }                                                                            \
     } while (0)
 
+// Launch of a kernel that may start while the kernel before it in the stream
+// still runs: its CTAs take their places and read what only the context holds,
+// then wait in after_previous_kernel() for that kernel's end and writes.  The
+// kernel before it lets it start with let_next_kernel_start().  Every CTA of
+// both has to pass after_previous_kernel() when it was itself launched so, so
+// that its end implies the end of what came before.  (early = false: a plain launch.)
+// An SM keeps its split of L1 and shared memory while CTAs are on it, so a
+// kernel that starts beside the tensor-core GEMM runs with the 28 KB of L1 that
+// its rings leave; the solves want more (262144 x 200 x 96: 919 us per step
+// plainly launched, 1002 early; temperatures only 211, 306).  They start early in calls
+// where the launch latency saved counts for more (early_solve; 16384 cells 105
+// -> 94 us, 32768 157 -> 154, 65536 274 -> 285).
+template <class... P, class... A>
+cudaError_t launch_early(bool early, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                         const A &...args) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+inline bool early_solve(int64_t cells, int num_sms, bool tc) { return !tc || cells <= 256 * (int64_t)num_sms; }
+__device__ __forceinline__ void after_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_kernel_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Kernels' entry points (host launchers), each returning a dust_status.
 // (zero, nzero: words the absorption kernel also clears, for counters of a
 // later kernel of the call)
@@ -337,14 +368,15 @@ void fill_emit_req(const dust_ctx *ctx, const EmitPlan &p, int64_t C, const Scra
 // With solved = true the temperatures, pairs and cell records are already
 // there (fused absorption + solve) and only the emission runs; with pass0 > 0
 // the grain passes before pass0 are done too (their sums carried in accp).
+// early: the solve may start beside the kernel before it (launch_early).
 int launch_emit_batch(EmitBatch &B, int num_sms, cudaStream_t st, cudaEvent_t between = nullptr,
-                      bool solved = false, int *nlaunch = nullptr, int pass0 = 0);
+                      bool solved = false, int *nlaunch = nullptr, int pass0 = 0, bool early = false);
 
 // Orders the cells of every request of the batch by the class of its key
-// (three launches: zero the counts, classify, scatter).  Cells of one class
+// (zero the counts, unless the absorption kernel has; classify; scatter).  Cells of one class
 // run together in the emission, so that the 32 lanes of a warp take the same
 // regime branches; the order never changes a result.
-int launch_order(OrderBatch &B, cudaStream_t st, int *nlaunch);
+int launch_order(OrderBatch &B, cudaStream_t st, int *nlaunch, bool zeroed = false);
 // Key of the ordering: the reference grain of a context.
 inline int order_ref_grain(int G) { return G / 2; }
 
@@ -353,7 +385,7 @@ inline int order_ref_grain(int G) { return G / 2; }
 // not apply) and the launch (for req.g1 = gc < G8 the first grain pass only).
 size_t plan_solve_emit(const dust_ctx *ctx, bool emit, bool mass, int *TC, int *gc);
 int launch_solve_emit_fused(const EmitReq &req, int TC, size_t smem, int num_sms, cudaStream_t st,
-                            int *nlaunch = nullptr);
+                            int *nlaunch = nullptr, bool early = false);
 
 // A small call's solve + emission with each tile's k-groups split over several
 // CTAs: the plan, and the launch (cnt: one zeroed counter per tile).

@@ -22,6 +22,7 @@ __global__ void __launch_bounds__(NTH, 2) k_gemm_simt(const __grid_constant__ Si
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
 
     const int64_t tile = blockIdx.x;
+    let_next_kernel_start();
     if (tile == 0)
         for (int i = tid; i < B.nzero; i += NTH) B.zero[i] = 0;
     int ri = 0;

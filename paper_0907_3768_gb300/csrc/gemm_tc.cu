@@ -319,6 +319,7 @@ __device__ __forceinline__ void gemm_body(const TcBatch &p, const SolveList *sl)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t ntiles = p.ntiles;
     const int nacc = p.nacc;
+    let_next_kernel_start();
     if (blockIdx.x == 0)
         for (int i = threadIdx.x; i < p.nzero; i += blockDim.x) p.zero[i] = 0;
 
@@ -637,6 +638,7 @@ __global__ void __launch_bounds__(NTHREADS_T, 1) k_gemm_tc_t(const __grid_consta
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t ntiles = p.ntiles;
+    let_next_kernel_start();
     if (blockIdx.x == 0)
         for (int i = threadIdx.x; i < p.nzero; i += blockDim.x) p.zero[i] = 0;
 

@@ -40,6 +40,8 @@ __device__ __forceinline__ int req_of_block(const OrderBatch &B, int blk) {
 }
 
 __global__ void __launch_bounds__(ORD_TH) k_order_zero(const __grid_constant__ OrderBatch B) {
+    let_next_kernel_start();
+    after_previous_kernel();
     unsigned *h = B.req[blockIdx.x].hist;
     for (int i = threadIdx.x; i < 2 * NBK; i += ORD_TH) h[i] = 0u;
 }
@@ -52,6 +54,8 @@ __global__ void __launch_bounds__(ORD_TH) k_order_classify(const __grid_constant
     const int64_t c0 = (int64_t)(blockIdx.x - q.block_begin) * ORD_CPB;
     const int64_t c1 = min(c0 + ORD_CPB, q.C);
     for (int i = threadIdx.x; i < NBK; i += ORD_TH) cnt[i] = 0u;
+    let_next_kernel_start();
+    after_previous_kernel();
     __syncthreads();
     for (int64_t c = c0 + threadIdx.x; c < c1; c += ORD_TH) {
         const int b = key_class(__ldg(q.key + c * q.kstride));
@@ -73,6 +77,8 @@ __global__ void __launch_bounds__(ORD_TH) k_order_scatter(const __grid_constant_
     const int64_t c0 = (int64_t)(blockIdx.x - q.block_begin) * ORD_CPB;
     const int64_t c1 = min(c0 + ORD_CPB, q.C);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    let_next_kernel_start();
+    after_previous_kernel();
     // exclusive scan of the NBK counts: four consecutive classes per thread
     constexpr int PER = NBK / ORD_TH;
     unsigned v[PER], s = 0;
@@ -109,7 +115,7 @@ __global__ void __launch_bounds__(ORD_TH) k_order_scatter(const __grid_constant_
 
 }  // namespace
 
-int launch_order(OrderBatch &B, cudaStream_t st, int *nlaunch) {
+int launch_order(OrderBatch &B, cudaStream_t st, int *nlaunch, bool zeroed) {
     if (nlaunch) *nlaunch = 0;
     int blocks = 0;
     for (int i = 0; i < B.nreq; ++i) {
@@ -118,13 +124,10 @@ int launch_order(OrderBatch &B, cudaStream_t st, int *nlaunch) {
     }
     B.nblocks = blocks;
     if (blocks == 0) return DUST_OK;
-    k_order_zero<<<B.nreq, ORD_TH, 0, st>>>(B);
-    DUST_CUDA_TRY(cudaGetLastError());
-    k_order_classify<<<blocks, ORD_TH, 0, st>>>(B);
-    DUST_CUDA_TRY(cudaGetLastError());
-    k_order_scatter<<<blocks, ORD_TH, 0, st>>>(B);
-    DUST_CUDA_TRY(cudaGetLastError());
-    if (nlaunch) *nlaunch = 3;
+    if (!zeroed) DUST_CUDA_TRY(launch_early(true, k_order_zero, B.nreq, ORD_TH, 0, st, B));
+    DUST_CUDA_TRY(launch_early(true, k_order_classify, blocks, ORD_TH, 0, st, B));
+    DUST_CUDA_TRY(launch_early(true, k_order_scatter, blocks, ORD_TH, 0, st, B));
+    if (nlaunch) *nlaunch = zeroed ? 2 : 3;
     return DUST_OK;
 }
 

@@ -107,6 +107,14 @@ int solve_view(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t 
     const SplitPlan split = fuse_emit ? plan_solve_emit_split(ctx, C, mass) : SplitPlan{};
     int *cnt = reinterpret_cast<int *>(sv.prep);
     const int ncnt = split.parts > 1 && resid ? (int)((C * split.lpc + 31) / 32) : 0;
+    // The emission order groups cells of like temperatures into the emission's
+    // 32-cell tiles; it never changes a result.  Small calls skip it: there the
+    // ordering's launches cost more than the warp-uniform regimes save.
+    const bool ordered = !split.parts && C > (int64_t)32 * ctx->num_sms && (L || resid) && sv.order && sv.bkt && sv.hist;
+    const bool order_now = ordered && !keep_order;
+    // (the absorption kernel also clears the class counts)
+    int *zero = order_now ? reinterpret_cast<int *>(sv.hist) : cnt;
+    const int nzero = order_now ? 2 * NBK : ncnt;
     int rc = DUST_OK;
     if (fused) {
         // one kernel through the temperatures: S stays in tensor memory
@@ -122,20 +130,16 @@ int solve_view(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t 
         if (rc == DUST_OK) rc = finish_tc_batch(tb, precision, ctx->smem_optin, &smem, true);
         if (rc == DUST_OK) rc = launch_tc_batch(tb, precision, smem, ctx->num_sms, st, &sl);
     } else {
-        rc = precision == DUST_PREC_FP32 ? launch_gemm_simt(ctx, C, J, ld, sv.S, st, cnt, ncnt)
-                                         : launch_gemm_tc(ctx, precision, C, J, ld, sv.S, st, cnt, ncnt);
+        rc = precision == DUST_PREC_FP32 ? launch_gemm_simt(ctx, C, J, ld, sv.S, st, zero, nzero)
+                                         : launch_gemm_tc(ctx, precision, C, J, ld, sv.S, st, zero, nzero);
     }
     if (rc == DUST_OK) nl_total += 1;
     int ftc = 0, fgc = 0;
     const size_t fsmem = fuse_emit && !split.parts ? plan_solve_emit(ctx, L || resid, mass, &ftc, &fgc) : 0;
     if (fsmem && fgc != p.gcp) return set_error(DUST_EINVAL, "internal: grain passes of the two emission forms differ");
-    // The emission order groups cells of like temperatures into the emission's
-    // 32-cell tiles; it never changes a result.  Small calls skip it: there the
-    // ordering's three launches cost more than the warp-uniform regimes save.
-    const bool ordered = !split.parts && C > (int64_t)32 * ctx->num_sms;
-    if (keep_order && (L || resid) && ordered && sv.order && sv.bkt && sv.hist) {
+    if (keep_order && ordered) {
         B.req[0].order = sv.order;
-    } else if (rc == DUST_OK && (L || resid) && ordered && sv.order && sv.bkt && sv.hist) {
+    } else if (rc == DUST_OK && order_now) {
         // emission order: cells classed by the absorbed power of the reference
         // grain (S), or by its inverse temperature where S stayed in tensor memory
         const int gref = order_ref_grain(ctx->G);
@@ -155,10 +159,11 @@ int solve_view(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t 
         o.hist = sv.hist;
         o.order = sv.order;
         int nl = 0;
-        rc = launch_order(ob, st, &nl);
+        rc = launch_order(ob, st, &nl, !fused);
         nl_total += nl;
         B.req[0].order = sv.order;
     }
+    const bool early = early_solve(C, ctx->num_sms, precision != DUST_PREC_FP32);
     if (rc == DUST_OK) {
         if (ev && ev[1]) DUST_CUDA_TRY(cudaEventRecord(ev[1], st));
         int nl = 0;
@@ -170,14 +175,14 @@ int solve_view(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t 
             // the solve runs inside the emission kernel: its time is reported with the emission's;
             // where the grains come in passes the kernel emits the first and k_emit the others
             if (ev && ev[2]) DUST_CUDA_TRY(cudaEventRecord(ev[2], st));
-            rc = launch_solve_emit_fused(B.req[0], ftc, fsmem, ctx->num_sms, st, &nl);
+            rc = launch_solve_emit_fused(B.req[0], ftc, fsmem, ctx->num_sms, st, &nl, early);
             if (rc == DUST_OK && fgc < (mass ? ctx->tbm : ctx->tb).G8) {
                 nl_total += nl;
                 nl = 0;
                 rc = launch_emit_batch(B, ctx->num_sms, st, nullptr, true, &nl, 1);
             }
         } else {
-            rc = launch_emit_batch(B, ctx->num_sms, st, ev ? ev[2] : nullptr, fused, &nl);
+            rc = launch_emit_batch(B, ctx->num_sms, st, ev ? ev[2] : nullptr, fused, &nl, 0, early);
         }
         nl_total += nl;
         if (ev && ev[3]) DUST_CUDA_TRY(cudaEventRecord(ev[3], st));

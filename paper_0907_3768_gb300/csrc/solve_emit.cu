@@ -221,6 +221,7 @@ __device__ __forceinline__ void solve_cell(const EmitReq &q, int64_t cell, int l
 template <int NB, bool TONLY>
 __global__ void __launch_bounds__(SOLVE_TH, TONLY ? solve_tonly_ctas(NB) : (NB >= 4 ? 5 : 6))
     k_solve(const __grid_constant__ EmitBatch B) {
+    after_previous_kernel();
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * SOLVE_TH) >> 5;
     int64_t u = ((int64_t)blockIdx.x * SOLVE_TH + threadIdx.x) >> 5;  // this warp's first cell
@@ -765,6 +766,7 @@ __global__ void __launch_bounds__(fse_th(PASS), 1) k_solve_emit(const __grid_con
         *claim = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    after_previous_kernel();
     __syncthreads();
 
     if (warp >= FE_W) {
@@ -904,6 +906,7 @@ __global__ void __launch_bounds__(SPL_TH, 2) k_solve_emit_split(const __grid_con
         sC[i + kg] = __ldg(src + i);  // rows of CST = 2 G8 + 1
     }
     if (tid == 0) *claim = 0;
+    after_previous_kernel();
     float s0[NB], n0[NB];
     if (warp < nc) load_pass<NB>(q, ordered_cell(q, c0 + warp), 0, lane, s0, n0);
     for (int cl = warp; cl < nc; cl += SPL_W) {
@@ -1076,7 +1079,7 @@ void fill_emit_req(const dust_ctx *ctx, const EmitPlan &p, int64_t C, const Scra
 // Numbers the cells and emission tiles of a filled batch; launches the solve
 // over every request, then the emission over the requests that want it.
 int launch_emit_batch(EmitBatch &B, int num_sms, cudaStream_t st, cudaEvent_t between,
-                      bool solved, int *nlaunch, int pass0) {
+                      bool solved, int *nlaunch, int pass0, bool early) {
     int nl = 0;
     int64_t cells = 0;
     for (int i = 0; i < B.nreq; ++i) {
@@ -1097,17 +1100,17 @@ int launch_emit_batch(EmitBatch &B, int num_sms, cudaStream_t st, cudaEvent_t be
         for (int i = 0; i < B.nreq; ++i) tonly = tonly && !(B.req[i].mode & EMIT_ON);
         if (tonly) {
             switch (nb) {
-                case 1: k_solve<1, true><<<(unsigned)grid, SOLVE_TH, 0, st>>>(B); break;
-                case 2: k_solve<2, true><<<(unsigned)grid, SOLVE_TH, 0, st>>>(B); break;
-                case 3: k_solve<3, true><<<(unsigned)grid, SOLVE_TH, 0, st>>>(B); break;
-                default: k_solve<4, true><<<(unsigned)grid, SOLVE_TH, 0, st>>>(B); break;
+                case 1: DUST_CUDA_TRY(launch_early(early, k_solve<1, true>, (unsigned)grid, SOLVE_TH, 0, st, B)); break;
+                case 2: DUST_CUDA_TRY(launch_early(early, k_solve<2, true>, (unsigned)grid, SOLVE_TH, 0, st, B)); break;
+                case 3: DUST_CUDA_TRY(launch_early(early, k_solve<3, true>, (unsigned)grid, SOLVE_TH, 0, st, B)); break;
+                default: DUST_CUDA_TRY(launch_early(early, k_solve<4, true>, (unsigned)grid, SOLVE_TH, 0, st, B)); break;
             }
         } else {
             switch (nb) {
-                case 1: k_solve<1, false><<<(unsigned)grid, SOLVE_TH, 0, st>>>(B); break;
-                case 2: k_solve<2, false><<<(unsigned)grid, SOLVE_TH, 0, st>>>(B); break;
-                case 3: k_solve<3, false><<<(unsigned)grid, SOLVE_TH, 0, st>>>(B); break;
-                default: k_solve<4, false><<<(unsigned)grid, SOLVE_TH, 0, st>>>(B); break;
+                case 1: DUST_CUDA_TRY(launch_early(early, k_solve<1, false>, (unsigned)grid, SOLVE_TH, 0, st, B)); break;
+                case 2: DUST_CUDA_TRY(launch_early(early, k_solve<2, false>, (unsigned)grid, SOLVE_TH, 0, st, B)); break;
+                case 3: DUST_CUDA_TRY(launch_early(early, k_solve<3, false>, (unsigned)grid, SOLVE_TH, 0, st, B)); break;
+                default: DUST_CUDA_TRY(launch_early(early, k_solve<4, false>, (unsigned)grid, SOLVE_TH, 0, st, B)); break;
             }
         }
         DUST_CUDA_TRY(cudaGetLastError());
@@ -1232,17 +1235,17 @@ size_t plan_solve_emit(const dust_ctx *ctx, bool emit, bool mass, int *TC, int *
 
 // The fused kernel over one request (general form), then the residual fold.
 template <bool MASS, bool PASS>
-int launch_fse(const EmitReq &r, int nb, unsigned grid, size_t smem, cudaStream_t st) {
+int launch_fse(const EmitReq &r, int nb, unsigned grid, size_t smem, bool early, cudaStream_t st) {
     const void *kern = nb == 1 ? reinterpret_cast<const void *>(k_solve_emit<1, MASS, PASS>)
                      : nb == 2 ? reinterpret_cast<const void *>(k_solve_emit<2, MASS, PASS>)
                      : nb == 3 ? reinterpret_cast<const void *>(k_solve_emit<3, MASS, PASS>)
                                : reinterpret_cast<const void *>(k_solve_emit<4, MASS, PASS>);
     DUST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     switch (nb) {
-        case 1: k_solve_emit<1, MASS, PASS><<<grid, fse_th(PASS), smem, st>>>(r); break;
-        case 2: k_solve_emit<2, MASS, PASS><<<grid, fse_th(PASS), smem, st>>>(r); break;
-        case 3: k_solve_emit<3, MASS, PASS><<<grid, fse_th(PASS), smem, st>>>(r); break;
-        default: k_solve_emit<4, MASS, PASS><<<grid, fse_th(PASS), smem, st>>>(r); break;
+        case 1: DUST_CUDA_TRY(launch_early(early, k_solve_emit<1, MASS, PASS>, grid, fse_th(PASS), smem, st, r)); break;
+        case 2: DUST_CUDA_TRY(launch_early(early, k_solve_emit<2, MASS, PASS>, grid, fse_th(PASS), smem, st, r)); break;
+        case 3: DUST_CUDA_TRY(launch_early(early, k_solve_emit<3, MASS, PASS>, grid, fse_th(PASS), smem, st, r)); break;
+        default: DUST_CUDA_TRY(launch_early(early, k_solve_emit<4, MASS, PASS>, grid, fse_th(PASS), smem, st, r)); break;
     }
     DUST_CUDA_TRY(cudaGetLastError());
     return DUST_OK;
@@ -1290,8 +1293,7 @@ int launch_split(const EmitReq &r, int nb, unsigned grid, const SplitPlan &p, in
     auto kern = nb == 1 ? k_solve_emit_split<1, MASS, LPC> : nb == 2 ? k_solve_emit_split<2, MASS, LPC>
               : nb == 3 ? k_solve_emit_split<3, MASS, LPC> : k_solve_emit_split<4, MASS, LPC>;
     DUST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem));
-    kern<<<grid, SPL_TH, p.smem, st>>>(r, p.parts, cnt);
-    DUST_CUDA_TRY(cudaGetLastError());
+    DUST_CUDA_TRY(launch_early(true, kern, grid, SPL_TH, p.smem, st, r, p.parts, cnt));
     return DUST_OK;
 }
 
@@ -1305,7 +1307,7 @@ int launch_solve_emit_split(const EmitReq &r, const SplitPlan &p, int *cnt, cuda
 }
 
 int launch_solve_emit_fused(const EmitReq &req, int TC, size_t smem, int num_sms, cudaStream_t st,
-                            int *nlaunch) {
+                            int *nlaunch, bool early) {
     if (nlaunch) *nlaunch = 0;
     if (req.C <= 0) return DUST_OK;
     EmitBatch E;
@@ -1327,8 +1329,8 @@ int launch_solve_emit_fused(const EmitReq &req, int TC, size_t smem, int num_sms
     const int nb = std::min(pass ? 3 : NB_MAX, (r.tb.G8 + 31) / 32);
     const bool mass = (r.mode & EMIT_MASS) != 0;
     const unsigned grid = (unsigned)std::min<int64_t>(E.ntiles, num_sms);
-    int rc = mass ? (pass ? launch_fse<true, true>(r, nb, grid, smem, st) : launch_fse<true, false>(r, nb, grid, smem, st))
-                  : (pass ? launch_fse<false, true>(r, nb, grid, smem, st) : launch_fse<false, false>(r, nb, grid, smem, st));
+    int rc = mass ? (pass ? launch_fse<true, true>(r, nb, grid, smem, early, st) : launch_fse<true, false>(r, nb, grid, smem, early, st))
+                  : (pass ? launch_fse<false, true>(r, nb, grid, smem, early, st) : launch_fse<false, false>(r, nb, grid, smem, early, st));
     if (rc != DUST_OK) return rc;
     if (nlaunch) *nlaunch = 1;  // the residual fold runs inside the kernel
     return DUST_OK;
