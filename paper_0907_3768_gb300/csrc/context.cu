@@ -429,6 +429,8 @@ void free_context(dust_ctx *ctx) {
     cudaFree(ctx->newton_grain);
     cudaFree(ctx->mass_mem);
     cudaFree(ctx->cpl);
+    if (ctx->cpl_host) cudaFreeHost(ctx->cpl_host);
+    if (ctx->cpl_ev) cudaEventDestroy(ctx->cpl_ev);
     cudaFree(ctx->fl_mem);
     auto &hs = ctx->hs;
     for (int i = 0; i < dust_ctx::NHB; ++i) {

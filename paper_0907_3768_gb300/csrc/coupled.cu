@@ -20,8 +20,8 @@ constexpr int CPL_TH = 128;
 
 // One warp per cell: the change of L against the previous iterate (folded
 // into *change with an integer max on the float's bits, exact for values
-// >= 0), then Lprev = L and Jw = J_ext + E L.  *next, the word of the
-// iteration after this one, is cleared here.
+// >= 0), then Lprev = L and Jw = J_ext + E L.  The last CTA to finish (count)
+// leaves the change in the host's word and clears both words for the next pass.
 // The pass is six rows per cell, bound by memory (by L2 up to some 30000
 // cells).  VEC (rows of whole, aligned 16-byte pieces): every load of a row is
 // issued before the first is used, which is once for K <= 256 (CPL_V pieces a
@@ -32,10 +32,11 @@ constexpr int CPL_V = 2;
 template <bool VEC>
 __global__ void __launch_bounds__(CPL_TH) k_couple(int64_t C, int K, int64_t ld, const float *Jext,
                                                    const float *E, const float *L, float *Lprev, float *Jw,
-                                                   int first, unsigned int *change, unsigned int *next) {
+                                                   int first, unsigned int *change, unsigned int *count,
+                                                   volatile unsigned int *host) {
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * CPL_TH) >> 5;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *next = 0u;
+    after_previous_kernel();
     for (int64_t c = ((int64_t)blockIdx.x * CPL_TH + threadIdx.x) >> 5; c < C; c += nw) {
         const float *Lr = L + c * ld;
         float *Pr = Lprev + c * ld;
@@ -88,6 +89,16 @@ __global__ void __launch_bounds__(CPL_TH) k_couple(int64_t C, int K, int64_t ld,
             float ch = d > 0.f ? (peak > 0.f ? d / peak : INFINITY) : 0.f;
             if (!(ch == ch)) ch = INFINITY;  // NaN counts as not converged
             atomicMax(change, __float_as_uint(ch));
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(count, 1u) == gridDim.x - 1) {
+            __threadfence();
+            *host = atomicExch(change, 0u);
+            *count = 0u;
+            __threadfence_system();
         }
     }
 }
@@ -166,33 +177,55 @@ extern "C" int dust_solve_coupled(dust_ctx *ctx, int64_t n_cells, const float *J
         cudaGetLastError();
         rc = set_error(DUST_ECUDA, "clearing the change words failed");
     }
-    while (rc == DUST_OK && it < max_iters) {
+    if (rc == DUST_OK && !ctx->cpl_host && cudaHostAlloc((void **)&ctx->cpl_host, sizeof(unsigned int), cudaHostAllocMapped) != cudaSuccess) {
+        cudaGetLastError();
+        ctx->cpl_host = nullptr;
+        rc = set_error(DUST_ENOMEM, "the coupled solve's page-locked word: cudaHostAlloc failed");
+    }
+    if (rc == DUST_OK && !ctx->cpl_ev && cudaEventCreateWithFlags(&ctx->cpl_ev, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        ctx->cpl_ev = nullptr;
+        rc = set_error(DUST_ECUDA, "the coupled solve's event could not be made");
+    }
+    // While the host learns a pass's change, the GPU runs the next pass's
+    // absorption, which writes nothing but scratch: the round trip (about 10 us)
+    // would leave it idle.  Not where absorption and solve are one kernel, nor
+    // while stages are timed.
+    const bool ahead = !(ctx->fused && precision != DUST_PREC_FP32) && !ctx->prof_on;
+    bool absorbed = false;
+    auto solve = [&](int phases) {
         // the cells' classes change little from one iterate to the next, and no
         // result depends on them: the emission order is made once (16384 cells x 200 x
         // 96, 24 solves: 3.39 ms with a new order for each, 3.06 with one)
-        rc = solve_device(ctx, precision, n_cells, Jcur, ld, n, T, L, resid, flags, ctx->S, st, false, it > 0);
+        return solve_device(ctx, precision, n_cells, Jcur, ld, n, T, L, resid, flags, ctx->S, st, false, it > 0, phases);
+    };
+    while (rc == DUST_OK && it < max_iters) {
+        rc = solve(absorbed ? SOLVE_REST : SOLVE_ALL);
+        absorbed = false;
         if (rc != DUST_OK) break;
         ++it;
-        unsigned int *now = chg + (it & 1), *next = chg + ((it + 1) & 1);
-        if (vec) k_couple<true><<<(unsigned)grid, CPL_TH, 0, st>>>(n_cells, ctx->K, ld, J_ext, E, L, Lprev, Jw, it == 1, now, next);
-        else k_couple<false><<<(unsigned)grid, CPL_TH, 0, st>>>(n_cells, ctx->K, ld, J_ext, E, L, Lprev, Jw, it == 1, now, next);
-        cudaError_t e = cudaGetLastError();
-        if (it == 1 && it < max_iters && e == cudaSuccess) {  // nothing to compare with yet: the next solve follows at once
-            Jcur = Jw;
-            continue;
+        cudaError_t e = launch_early(true, vec ? k_couple<true> : k_couple<false>, (unsigned)grid, CPL_TH, 0, st, n_cells, ctx->K, ld,
+                                     J_ext, E, (const float *)L, Lprev, Jw, (int)(it == 1), chg, chg + 1,
+                                     (volatile unsigned int *)ctx->cpl_host);
+        Jcur = Jw;
+        if (it == 1 && it < max_iters && e == cudaSuccess) continue;  // nothing to compare with yet: the next solve follows at once
+        if (e == cudaSuccess) e = cudaEventRecord(ctx->cpl_ev, st);
+        if (e == cudaSuccess && ahead && it < max_iters) {
+            rc = solve(SOLVE_ABSORB);
+            absorbed = rc == DUST_OK;
         }
-        unsigned int bits = 0;
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&bits, now, sizeof(bits), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) {
-            rc = set_error(DUST_ECUDA, "coupled iteration: %s", cudaGetErrorString(e));
-            break;
-        }
+        if (e == cudaSuccess) e = cudaEventSynchronize(ctx->cpl_ev);
+        if (e != cudaSuccess && rc == DUST_OK) rc = set_error(DUST_ECUDA, "coupled iteration: %s", cudaGetErrorString(e));
+        if (rc != DUST_OK) break;
         if (it > 1) {
+            const unsigned int bits = *(volatile unsigned int *)ctx->cpl_host;
             std::memcpy(&change, &bits, sizeof(change));
             if (change <= tol) break;
         }
-        Jcur = Jw;
+    }
+    if (absorbed && cudaStreamSynchronize(st) != cudaSuccess && rc == DUST_OK) {
+        cudaGetLastError();
+        rc = set_error(DUST_ECUDA, "coupled iteration: waiting for the last absorption failed");
     }
     if (prev >= 0 && prev != ctx->device) cudaSetDevice(prev);
     if (iters_done) *iters_done = it;

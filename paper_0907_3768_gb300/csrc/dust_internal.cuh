@@ -253,6 +253,9 @@ struct dust_ctx {
     // working J, previous L and a change word of dust_solve_coupled
     void *cpl = nullptr;
     size_t cpl_bytes = 0;
+    // page-locked word where k_couple leaves the change, and the event after it
+    unsigned int *cpl_host = nullptr;
+    cudaEvent_t cpl_ev = nullptr;
     // scratch of scaled absorbed powers S[C][Gs]
     float *S = nullptr;
     size_t S_cap = 0;         // in cells
@@ -392,6 +395,8 @@ int launch_solve_emit_fused(const EmitReq &req, int TC, size_t smem, int num_sms
 SplitPlan plan_solve_emit_split(const dust_ctx *ctx, int64_t C, bool mass);
 int launch_solve_emit_split(const EmitReq &r, const SplitPlan &p, int *cnt, cudaStream_t st);
 
+enum SolvePhase { SOLVE_ABSORB = 1, SOLVE_REST = 2, SOLVE_ALL = 3 };
+
 // Grow the context's scratch to hold `cells` cells (synchronises `st` first).
 int ensure_scratch(dust_ctx *ctx, int64_t cells, cudaStream_t st);
 
@@ -401,14 +406,16 @@ int ensure_scratch(dust_ctx *ctx, int64_t cells, cudaStream_t st);
 // ev (optional, four events) marks absorption / solve / emission boundaries.
 // keep_order: the scratch still holds the emission order that the last call
 // made for as many cells; it is taken as it is.
+// phases: the absorption alone (it writes the scratch only; not where
+// ctx->fused), or what follows it, in two calls with otherwise the same arguments.
 int solve_view(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t ld, const float *n, float *T,
                float *L, double *resid, uint8_t *flags, const ScratchView &sv, cudaStream_t st, bool mass,
-               int *nlaunch, cudaEvent_t *ev = nullptr, bool keep_order = false);
+               int *nlaunch, cudaEvent_t *ev = nullptr, bool keep_order = false, int phases = SOLVE_ALL);
 // The whole path on device buffers with scratch of scratch_bytes(ctx, C, true)
 // bytes at `scratch`.
 int solve_device(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t ld,
                  const float *n, float *T, float *L, double *resid, uint8_t *flags, void *scratch,
-                 cudaStream_t st, bool mass = false, bool keep_order = false);
+                 cudaStream_t st, bool mass = false, bool keep_order = false, int phases = SOLVE_ALL);
 
 // Bounded spin budget for device-side waits: a wait that exceeds it records
 // DUST_ETIMEOUT in the status word and gives up.

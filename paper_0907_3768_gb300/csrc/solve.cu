@@ -90,7 +90,7 @@ cudaEvent_t prof_event(dust_ctx *ctx) {
 
 int solve_view(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t ld, const float *n, float *T,
                float *L, double *resid, uint8_t *flags, const ScratchView &sv, cudaStream_t st, bool mass,
-               int *nlaunch, cudaEvent_t *ev, bool keep_order) {
+               int *nlaunch, cudaEvent_t *ev, bool keep_order, int phases) {
     int nl_total = 0;
     if (nlaunch) *nlaunch = 0;
     if (C == 0) return DUST_OK;
@@ -129,11 +129,15 @@ int solve_view(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t 
         rc = make_tc_req(ctx, precision, C, J, ld, sv.S, tb.req[0], tb.tm[0]);
         if (rc == DUST_OK) rc = finish_tc_batch(tb, precision, ctx->smem_optin, &smem, true);
         if (rc == DUST_OK) rc = launch_tc_batch(tb, precision, smem, ctx->num_sms, st, &sl);
-    } else {
+    } else if (phases & SOLVE_ABSORB) {
         rc = precision == DUST_PREC_FP32 ? launch_gemm_simt(ctx, C, J, ld, sv.S, st, zero, nzero)
                                          : launch_gemm_tc(ctx, precision, C, J, ld, sv.S, st, zero, nzero);
     }
-    if (rc == DUST_OK) nl_total += 1;
+    if (rc == DUST_OK && (fused || (phases & SOLVE_ABSORB))) nl_total += 1;
+    if (!(phases & SOLVE_REST)) {
+        if (nlaunch) *nlaunch = nl_total;
+        return rc;
+    }
     int ftc = 0, fgc = 0;
     const size_t fsmem = fuse_emit && !split.parts ? plan_solve_emit(ctx, L || resid, mass, &ftc, &fgc) : 0;
     if (fsmem && fgc != p.gcp) return set_error(DUST_EINVAL, "internal: grain passes of the two emission forms differ");
@@ -193,7 +197,7 @@ int solve_view(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t 
 
 int solve_device(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t ld, const float *n,
                  float *T, float *L, double *resid, uint8_t *flags, void *scratch, cudaStream_t st, bool mass,
-                 bool keep_order) {
+                 bool keep_order, int phases) {
     if (C == 0) return DUST_OK;
     const ScratchView sv = scratch_view(ctx, C, scratch);
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -201,7 +205,7 @@ int solve_device(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_
         for (int i = 0; i < 4; ++i) ev[i] = prof_event(ctx);
     const bool prof = ev[0] && ev[1] && ev[2] && ev[3];
     int nl = 0;
-    const int rc = solve_view(ctx, precision, C, J, ld, n, T, L, resid, flags, sv, st, mass, &nl, prof ? ev : nullptr, keep_order);
+    const int rc = solve_view(ctx, precision, C, J, ld, n, T, L, resid, flags, sv, st, mass, &nl, prof ? ev : nullptr, keep_order, phases);
     ctx->launches += (uint64_t)nl;
     for (int i = 0; i < 4; ++i) {
         if (!ev[i]) continue;

@@ -729,6 +729,7 @@ __device__ __forceinline__ int fse_tile(int it, int nb) {
 template <int NB, bool MASS, bool PASS>
 __global__ void __launch_bounds__(fse_th(PASS), 1) k_solve_emit(const __grid_constant__ EmitReq q) {
     constexpr int FE_W = fe_w(PASS), FS_W = fs_w(PASS), FSE_TH = fse_th(PASS);
+    let_next_kernel_start();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const DevTables &tb = q.tb;
     const int G8 = tb.G8, NKG = tb.NKG;
@@ -886,6 +887,7 @@ constexpr int SPL_TH = SPL_W * 32;
 template <int NB, bool MASS, int LPC>
 __global__ void __launch_bounds__(SPL_TH, 2) k_solve_emit_split(const __grid_constant__ EmitReq q, int parts, int *cnt) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    let_next_kernel_start();
     constexpr int TC = FSE_TC / LPC, PW = MASS ? 1 : 2, NP = 4 / LPC;
     const DevTables &tb = q.tb;
     const int G8 = tb.G8, NKG = tb.NKG, CST = 2 * G8 + 1, PS = G8 + 1;
