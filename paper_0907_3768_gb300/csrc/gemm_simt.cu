@@ -2,9 +2,18 @@
 //   S[c,g] = sum_k J[c,k] W32[g,k]                          (Eq. 6, scaled)
 // The paper's kernel 2 is the same matrix product with shared-memory tiles
 // over wavelength intervals (Section 4.2).  Here: 128-cell x (16 TN)-grain CTA
-// tiles over a work list of requests, 16-wavelength double-buffered stages,
-// an 8 x TN register tile per thread, FP32 FMA accumulation in ascending k
-// (so a cell's result does not depend on the tiling or the batch).
+// tiles over a work list of requests, stages of 16 wavelengths, an 8 x TN
+// register tile per thread, FP32 FMA accumulation in ascending k (so a cell's
+// result does not depend on the tiling or the batch).
+//
+// FMA-bound: at K = 200, G = 96 48 us of FMAs against 17 us of memory for 100000
+// cells.  Stages are filled by cp.async, a word at a time with the lanes along
+// k: rows of J may start anywhere (ld is the caller's), and 16 lanes read 64
+// consecutive bytes of one whatever its alignment.  (Loads through registers,
+// eight words of a row per thread, touched 32 lines per instruction when ld was
+// odd: 100003 x 201 x 96 took 119 us, now 98, 262144 x 200 x 96 254, now 217.)  Three CTAs
+// per SM up to 96 columns (two: 101 and 225 us).  A thread's columns come in
+// pairs, one 8-byte load and one packed FMA each (scalar FMAs: 112 and 251 us).
 #include "dust_internal.cuh"
 
 #include <algorithm>
@@ -12,13 +21,20 @@
 namespace dust {
 namespace {
 
-constexpr int BM = 128, BK = 16, NTH = 256;
+constexpr int BM = 128, BK = 16, NTH = 256, NST = 3;
+constexpr int AST = BM + 4;                                  // row of a stage of J: [BK][AST], 16-byte aligned
+__host__ __device__ constexpr int bst(int TN) { return 16 * TN + 2; }  // and of W: [BK][bst], even
+__host__ __device__ constexpr int stage_floats(int TN) { return BK * (AST + bst(TN)); }
+
+// A word to shared memory; 0 where `on` is false (nothing is read then).
+__device__ __forceinline__ void cp_word(uint32_t dst, const float *src, bool on) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(on ? 4 : 0) : "memory");
+}
 
 template <int TN>
-__global__ void __launch_bounds__(NTH, 2) k_gemm_simt(const __grid_constant__ SimtBatch B) {
-    constexpr int BN = 16 * TN;
-    __shared__ __align__(16) float As[2][BK][BM + 4];
-    __shared__ float Bs[2][BK][BN + 1];
+__global__ void __launch_bounds__(NTH, TN <= 6 ? 3 : 2) k_gemm_simt(const __grid_constant__ SimtBatch B) {
+    constexpr int BN = 16 * TN, NP = TN / 2, BST = bst(TN);
+    extern __shared__ __align__(16) float sm[];  // [NST] stages of J, then of W
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
 
     const int64_t tile = blockIdx.x;
@@ -33,88 +49,97 @@ __global__ void __launch_bounds__(NTH, 2) k_gemm_simt(const __grid_constant__ Si
     const int n0 = (int)(local % q.ntn) * BN;
     const int K = q.K, Kw = q.Kw, Gs = q.Gs;
     const int64_t C = q.C, ld = q.ld;
-    const float *__restrict__ W = q.W;
-    const bool vec = (ld % 4 == 0) && (((uintptr_t)q.J & 15) == 0);
 
-    // A loader: row ar, 8 consecutive k from ak
-    const int ar = tid >> 1, ak = (tid & 1) * 8;
-    const int64_t arow = m0 + ar;
-    const bool arow_ok = arow < C;
-    const float *__restrict__ Jrow = q.J + (arow_ok ? arow : 0) * ld;
-
-    float a_reg[8];
-    float b_reg[(BN * BK + NTH - 1) / NTH];
-
-    auto load_tile = [&](int k0) {
-        if (vec && arow_ok && k0 + ak + 8 <= K) {
-            float4 v0 = __ldg(reinterpret_cast<const float4 *>(Jrow + k0 + ak));
-            float4 v1 = __ldg(reinterpret_cast<const float4 *>(Jrow + k0 + ak + 4));
-            a_reg[0] = v0.x; a_reg[1] = v0.y; a_reg[2] = v0.z; a_reg[3] = v0.w;
-            a_reg[4] = v1.x; a_reg[5] = v1.y; a_reg[6] = v1.z; a_reg[7] = v1.w;
+    // this thread's words of a stage: wavelength tx of rows ty, ty + 16, ... of J
+    // and of W.  Rows past the last are the last again (nothing of them is
+    // stored), so that only wavelengths past K need a test, in the last stage.
+    const int64_t jrows = min(C - m0, (int64_t)BM);
+    const int wrows = min(Gs - n0, BN);
+    const float *jp = q.J + m0 * ld + tx, *wp = q.W + (size_t)n0 * Kw + tx;
+    const uint32_t sA = (uint32_t)__cvta_generic_to_shared(sm) + (tx * AST + ty) * 4;
+    const uint32_t sB = (uint32_t)__cvta_generic_to_shared(sm) + (BK * AST + tx * BST + ty) * 4;
+    auto load = [&](int t) {
+        const uint32_t off = (uint32_t)(t % NST * stage_floats(TN) * 4);
+        const bool on = t * BK + tx < K;
+        const float *j = on ? jp + t * BK : q.J, *w = wp + t * BK;  // W's rows are padded with zeros to Kw
+        if (jrows == BM) {
+            const float *r = j + (on ? ty * ld : 0);
+            const int64_t step = on ? 16 * ld : 0;
+#pragma unroll
+            for (int i = 0; i < BM / 16; ++i, r += step) cp_word(sA + off + 64 * i, r, on);
         } else {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                int k = k0 + ak + e;
-                a_reg[e] = (arow_ok && k < K) ? __ldg(Jrow + k) : 0.f;
-            }
+#pragma unroll 1
+            for (int i = 0; i < BM / 16; ++i) cp_word(sA + off + 64 * i, on ? j + min(ty + 16 * i, (int)jrows - 1) * ld : j, on);
         }
+        if (wrows == BN) {
+            const float *r = w + (size_t)ty * Kw;
 #pragma unroll
-        for (int i = 0; i < (BN * BK + NTH - 1) / NTH; ++i) {
-            int idx = tid + i * NTH;
-            int r = idx / BK, kk = idx % BK;
-            int g = n0 + r;
-            b_reg[i] = (idx < BN * BK && g < Gs) ? __ldg(W + (size_t)g * Kw + k0 + kk) : 0.f;
-        }
-    };
-    auto store_tile = [&](int buf) {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) As[buf][ak + e][ar] = a_reg[e];
-#pragma unroll
-        for (int i = 0; i < (BN * BK + NTH - 1) / NTH; ++i) {
-            int idx = tid + i * NTH;
-            if (idx < BN * BK) Bs[buf][idx % BK][idx / BK] = b_reg[i];
+            for (int i = 0; i < TN; ++i, r += 16 * Kw) cp_word(sB + off + 64 * i, r, true);
+        } else {
+#pragma unroll 1
+            for (int i = 0; i < TN; ++i) cp_word(sB + off + 64 * i, w + (size_t)min(ty + 16 * i, wrows - 1) * Kw, true);
         }
     };
 
-    float acc[8][TN];
+    // columns 32 p + 2 tx, 32 p + 2 tx + 1 for p < NP, and 32 NP + tx when TN is odd
+    float2 acc[8][NP > 0 ? NP : 1];
+    float last[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < 8; ++i) {
+        last[i] = 0.f;
 #pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
+        for (int p = 0; p < NP; ++p) acc[i][p] = make_float2(0.f, 0.f);
+    }
 
     const int nk = (K + BK - 1) / BK;
-    load_tile(0);
-    store_tile(0);
-    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < NST - 1; ++t) {
+        if (t < nk) load(t);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
     for (int t = 0; t < nk; ++t) {
-        const int buf = t & 1;
-        if (t + 1 < nk) load_tile((t + 1) * BK);
+        asm volatile("cp.async.wait_group %0;" ::"n"(NST - 2) : "memory");
+        __syncthreads();  // stage t is there for all, and stage t - 1 is read by all
+        if (t + NST - 1 < nk) load(t + NST - 1);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        const float *As = sm + t % NST * stage_floats(TN), *Bs = As + BK * AST;
 #pragma unroll
         for (int kk = 0; kk < BK; ++kk) {
-            float4 a0 = *reinterpret_cast<const float4 *>(&As[buf][kk][ty * 8]);
-            float4 a1 = *reinterpret_cast<const float4 *>(&As[buf][kk][ty * 8 + 4]);
-            float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            float b[TN];
+            const float4 a0 = *reinterpret_cast<const float4 *>(As + kk * AST + ty * 8);
+            const float4 a1 = *reinterpret_cast<const float4 *>(As + kk * AST + ty * 8 + 4);
+            const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
 #pragma unroll
-            for (int j = 0; j < TN; ++j) b[j] = Bs[buf][kk][tx + 16 * j];
+            for (int p = 0; p < NP; ++p) {
+                const float2 b = *reinterpret_cast<const float2 *>(Bs + kk * BST + 32 * p + 2 * tx);
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
+                for (int i = 0; i < 8; ++i) acc[i][p] = __ffma2_rn(make_float2(a[i], a[i]), b, acc[i][p]);
+            }
+            if (TN & 1) {
+                const float b = Bs[kk * BST + 32 * NP + tx];
 #pragma unroll
-                for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+                for (int i = 0; i < 8; ++i) last[i] = fmaf(a[i], b, last[i]);
+            }
         }
-        if (t + 1 < nk) store_tile(buf ^ 1);
-        __syncthreads();
     }
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-        int64_t row = m0 + ty * 8 + i;
+        const int64_t row = m0 + ty * 8 + i;
         if (row >= C) break;
+        float *out = q.S + row * Gs + n0;  // Gs and n0 are multiples of 16
 #pragma unroll
-        for (int j = 0; j < TN; ++j) {
-            int col = n0 + tx + 16 * j;
-            if (col < Gs) q.S[row * Gs + col] = acc[i][j];
-        }
+        for (int p = 0; p < NP; ++p)
+            if (n0 + 32 * p + 2 * tx < Gs) *reinterpret_cast<float2 *>(out + 32 * p + 2 * tx) = acc[i][p];
+        if ((TN & 1) && n0 + 32 * NP + tx < Gs) out[32 * NP + tx] = last[i];
     }
+}
+
+template <int TN>
+int launch_simt(const SimtBatch &B, unsigned grid, cudaStream_t st) {
+    constexpr int smem = NST * stage_floats(TN) * (int)sizeof(float);
+    DUST_CUDA_TRY(cudaFuncSetAttribute(k_gemm_simt<TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    k_gemm_simt<TN><<<grid, NTH, smem, st>>>(B);
+    DUST_CUDA_TRY(cudaGetLastError());
+    return DUST_OK;
 }
 
 }  // namespace
@@ -152,17 +177,15 @@ int launch_simt_batch(SimtBatch &B, cudaStream_t st) {
     if (t > 0x7fffffff) return set_error(DUST_EINVAL, "too many cells for one launch");
     const unsigned grid = (unsigned)t;
     switch (TN) {
-        case 1: k_gemm_simt<1><<<grid, NTH, 0, st>>>(B); break;
-        case 2: k_gemm_simt<2><<<grid, NTH, 0, st>>>(B); break;
-        case 3: k_gemm_simt<3><<<grid, NTH, 0, st>>>(B); break;
-        case 4: k_gemm_simt<4><<<grid, NTH, 0, st>>>(B); break;
-        case 5: k_gemm_simt<5><<<grid, NTH, 0, st>>>(B); break;
-        case 6: k_gemm_simt<6><<<grid, NTH, 0, st>>>(B); break;
-        case 7: k_gemm_simt<7><<<grid, NTH, 0, st>>>(B); break;
-        default: k_gemm_simt<8><<<grid, NTH, 0, st>>>(B); break;
+        case 1: return launch_simt<1>(B, grid, st);
+        case 2: return launch_simt<2>(B, grid, st);
+        case 3: return launch_simt<3>(B, grid, st);
+        case 4: return launch_simt<4>(B, grid, st);
+        case 5: return launch_simt<5>(B, grid, st);
+        case 6: return launch_simt<6>(B, grid, st);
+        case 7: return launch_simt<7>(B, grid, st);
+        default: return launch_simt<8>(B, grid, st);
     }
-    DUST_CUDA_TRY(cudaGetLastError());
-    return DUST_OK;
 }
 
 int launch_gemm_simt(const dust_ctx *ctx, int64_t C, const float *J, int64_t ld, float *S, cudaStream_t st,
