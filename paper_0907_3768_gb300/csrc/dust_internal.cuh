@@ -169,6 +169,13 @@ struct SplitPlan {
     size_t smem;
 };
 
+// Words that an absorption kernel clears for later kernels of its call: the
+// class counts of the ordering, the counters of a small call's parts.
+struct ZeroSpans {
+    int *p[2];
+    int n[2];
+};
+
 // One request of the tensor-core absorption kernel (its TMA descriptor for J
 // sits in TcBatch::tm at the same index).
 struct TcReq {
@@ -188,8 +195,7 @@ struct TcBatch {
     int orient;  // 0: cells are the MMA's M (128-cell tiles); 1: cells are its N (bn-cell tiles, Gs <= 128)
     int bn;      // orient 1: cells per tile (tc_tile_cells, set before the requests are made)
     int *status;
-    int *zero;      // nzero words to clear for a later kernel of the same call (or nzero = 0)
-    int nzero;
+    ZeroSpans zero;  // cleared for later kernels of the same call
 };
 
 // One request of the FP32 SIMT absorption kernel.
@@ -204,8 +210,7 @@ struct SimtBatch {
     SimtReq req[MAXREQ];
     int nreq;
     int64_t ntiles;
-    int *zero;      // as TcBatch's
-    int nzero;
+    ZeroSpans zero;
 };
 
 }  // namespace dust
@@ -332,12 +337,11 @@ __device__ __forceinline__ void after_previous_kernel() { asm volatile("griddepc
 __device__ __forceinline__ void let_next_kernel_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Kernels' entry points (host launchers), each returning a dust_status.
-// (zero, nzero: words the absorption kernel also clears, for counters of a
-// later kernel of the call)
+// (zero: words the absorption kernel also clears)
 int launch_gemm_simt(const dust_ctx *ctx, int64_t C, const float *J, int64_t ld, float *S,
-                     cudaStream_t st, int *zero = nullptr, int nzero = 0);
+                     cudaStream_t st, const ZeroSpans &zero = ZeroSpans{});
 int launch_gemm_tc(const dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t ld,
-                   float *S, cudaStream_t st, int *zero = nullptr, int nzero = 0);
+                   float *S, cudaStream_t st, const ZeroSpans &zero = ZeroSpans{});
 int launch_solve_emit(const dust_ctx *ctx, int64_t C, const ScratchView &sv, const float *n, float *T,
                       float *L, int64_t ld, double *resid, uint8_t *flags, cudaStream_t st, int *nlaunch = nullptr);
 EmitPlan plan_emit(const dust_ctx *ctx, bool emit, bool mass);
@@ -425,6 +429,13 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
+}
+
+// One CTA's threads clear the spans.
+__device__ __forceinline__ void clear_spans(const ZeroSpans &z) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        for (int i = threadIdx.x; i < z.n[k]; i += blockDim.x) z.p[k][i] = 0;
 }
 
 __device__ __forceinline__ void record_status(int *status, int code) {

@@ -39,8 +39,7 @@ __global__ void __launch_bounds__(NTH, TN <= 6 ? 3 : 2) k_gemm_simt(const __grid
 
     const int64_t tile = blockIdx.x;
     let_next_kernel_start();
-    if (tile == 0)
-        for (int i = tid; i < B.nzero; i += NTH) B.zero[i] = 0;
+    if (tile == 0) clear_spans(B.zero);
     int ri = 0;
     while (ri + 1 < B.nreq && tile >= B.req[ri + 1].tile_begin) ++ri;
     const SimtReq &q = B.req[ri];
@@ -189,12 +188,11 @@ int launch_simt_batch(SimtBatch &B, cudaStream_t st) {
 }
 
 int launch_gemm_simt(const dust_ctx *ctx, int64_t C, const float *J, int64_t ld, float *S, cudaStream_t st,
-                     int *zero, int nzero) {
+                     const ZeroSpans &zero) {
     if (C <= 0) return DUST_OK;
     SimtBatch B;
     B.nreq = 1;
     B.zero = zero;
-    B.nzero = nzero;
     make_simt_req(ctx, C, J, ld, S, B.req[0]);
     return launch_simt_batch(B, st);
 }

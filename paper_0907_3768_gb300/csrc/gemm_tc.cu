@@ -320,8 +320,7 @@ __device__ __forceinline__ void gemm_body(const TcBatch &p, const SolveList *sl)
     const int64_t ntiles = p.ntiles;
     const int nacc = p.nacc;
     let_next_kernel_start();
-    if (blockIdx.x == 0)
-        for (int i = threadIdx.x; i < p.nzero; i += blockDim.x) p.zero[i] = 0;
+    if (blockIdx.x == 0) clear_spans(p.zero);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.ns1; ++s) { mbar_init(&full1[s], 1); mbar_init(&empty1[s], 4); }
@@ -639,8 +638,7 @@ __global__ void __launch_bounds__(NTHREADS_T, 1) k_gemm_tc_t(const __grid_consta
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t ntiles = p.ntiles;
     let_next_kernel_start();
-    if (blockIdx.x == 0)
-        for (int i = threadIdx.x; i < p.nzero; i += blockDim.x) p.zero[i] = 0;
+    if (blockIdx.x == 0) clear_spans(p.zero);
 
     // W rows past Gs stay zero: the bulk copies write only the first Gs rows of each part
     for (int i = threadIdx.x; i < p.ns2 * 2 * WA_PART / 16; i += blockDim.x)
@@ -1033,12 +1031,11 @@ int launch_tc_batch(const TcBatch &B, int precision, size_t smem, int num_sms, c
 }
 
 int launch_gemm_tc(const dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t ld, float *S,
-                   cudaStream_t st, int *zero, int nzero) {
+                   cudaStream_t st, const ZeroSpans &zero) {
     if (C <= 0) return DUST_OK;
     TcBatch B;
     B.nreq = 1;
     B.zero = zero;
-    B.nzero = nzero;
     B.status = ctx->tb.status;
     B.orient = tc_orient(ctx);
     B.bn = tc_tile_cells(C, ctx->num_sms);

@@ -293,7 +293,7 @@ int launch_round(dust_server *s, const Round &rd) {
         if (prec == DUST_PREC_FP32) {
             SimtBatch B;
             B.nreq = 0;
-            B.nzero = 0;
+            B.zero = ZeroSpans{};
             for (size_t k = 0; k < parts.size(); ++k) {
                 const Part &p = parts[k];
                 if (p.r->precision != prec) continue;
@@ -311,7 +311,7 @@ int launch_round(dust_server *s, const Round &rd) {
             for (int orient = 0; orient < 2; ++orient) {
                 TcBatch B;
                 B.nreq = 0;
-                B.nzero = 0;
+                B.zero = ZeroSpans{};
                 B.status = nullptr;
                 B.orient = orient;
                 int64_t cells = 0;

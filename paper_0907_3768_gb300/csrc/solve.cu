@@ -108,19 +108,21 @@ int solve_view(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t 
     int *cnt = reinterpret_cast<int *>(sv.prep);
     const int ncnt = split.parts > 1 && resid ? (int)((C * split.lpc + 31) / 32) : 0;
     // The emission order groups cells of like temperatures into the emission's
-    // 32-cell tiles; it never changes a result.  Small calls skip it: there the
-    // ordering's launches cost more than the warp-uniform regimes save.
-    const bool ordered = !split.parts && C > (int64_t)32 * ctx->num_sms && (L || resid) && sv.order && sv.bkt && sv.hist;
+    // tiles; it never changes a result.  Calls of few cells, or of few Planck
+    // terms in the small-call kernel, skip it: there its two launches (some 10
+    // us) cost more than the warp-uniform regimes save, about a third of the
+    // emission (500 x 240: 512 cells 67 us without and 62 with it, 4864 cells
+    // 310 and 235; 350 x 96, 1024 cells 35 us without).
+    const bool ordered = (split.parts ? (double)C * ctx->K * ctx->G > 5e7 : C > (int64_t)32 * ctx->num_sms) && (L || resid) &&
+                         sv.order && sv.bkt && sv.hist;
     const bool order_now = ordered && !keep_order;
-    // (the absorption kernel also clears the class counts)
-    int *zero = order_now ? reinterpret_cast<int *>(sv.hist) : cnt;
-    const int nzero = order_now ? 2 * NBK : ncnt;
+    const ZeroSpans zero = {{reinterpret_cast<int *>(sv.hist), cnt}, {order_now ? 2 * NBK : 0, ncnt}};
     int rc = DUST_OK;
     if (fused) {
         // one kernel through the temperatures: S stays in tensor memory
         TcBatch tb;
         tb.nreq = 1;
-        tb.nzero = 0;
+        tb.zero = ZeroSpans{};
         tb.status = ctx->tb.status;
         tb.orient = 0;
         SolveList sl;
@@ -130,8 +132,8 @@ int solve_view(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t 
         if (rc == DUST_OK) rc = finish_tc_batch(tb, precision, ctx->smem_optin, &smem, true);
         if (rc == DUST_OK) rc = launch_tc_batch(tb, precision, smem, ctx->num_sms, st, &sl);
     } else if (phases & SOLVE_ABSORB) {
-        rc = precision == DUST_PREC_FP32 ? launch_gemm_simt(ctx, C, J, ld, sv.S, st, zero, nzero)
-                                         : launch_gemm_tc(ctx, precision, C, J, ld, sv.S, st, zero, nzero);
+        rc = precision == DUST_PREC_FP32 ? launch_gemm_simt(ctx, C, J, ld, sv.S, st, zero)
+                                         : launch_gemm_tc(ctx, precision, C, J, ld, sv.S, st, zero);
     }
     if (rc == DUST_OK && (fused || (phases & SOLVE_ABSORB))) nl_total += 1;
     if (!(phases & SOLVE_REST)) {

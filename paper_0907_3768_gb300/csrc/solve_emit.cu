@@ -1260,13 +1260,15 @@ SplitPlan plan_solve_emit_split(const dust_ctx *ctx, int64_t C, bool mass) {
     const DevTables &tb = mass ? ctx->tbm : ctx->tb;
     SplitPlan p{};
     const int64_t sms = ctx->num_sms;
-    // Where the fused kernel takes over.  It needs tiles of like temperatures, so
-    // the cell ordering (three launches, 16 us), and whole tiles for every SM; a
-    // small call is emitted unordered, which costs about half as much again per
-    // term.  Times per call of the fused kernel and of this one, in us: 200 x 96,
-    // 4900 cells 73 / 66, 7000 76 / 70, 8192 77 / 86, 9728 76 / 80; 64 x 16, 9728
-    // cells 38 / 22, 12288 43 / 29; 500 x 240, 4900 cells 354 / 303, 7000 369 / 425.
-    if (C > 40 * sms && (C > 96 * sms || (double)C * tb.K * tb.G > 1.5e8)) return p;
+    // Where the fused kernel takes over: it solves a tile while it emits another,
+    // but wants whole tiles for every SM.  Times per call of the fused kernel
+    // and of this one, in us: 200 x 96, 7000 cells 64 / 61, 8192 64 / 65; 350 x
+    // 96, 7000 cells 88 / 98, 8192 89 / 123; 64 x 16, 9728 cells 38 / 22, 12288
+    // 43 / 29.  Where its weights need grain passes (500 x 240) this one, which
+    // splits them by wavelength, stays ahead longer: 7000 cells 357 / 318, 8192
+    // 363 / 365, 9728 370 / 425.
+    const bool passes = plan_emit(ctx, true, mass).gcp < tb.G8;
+    if (C > 32 * sms && (passes ? C > 52 * sms : C > 96 * sms || (double)C * tb.K * tb.G > 1.4e8)) return p;
     // Four lanes per cell while tiles of 8 cells make at most two CTAs per SM, the
     // most that run at once; then two.  (200 x 96, in us with 1, 2 and 4 lanes: 32
     // cells 35 / 29 / 25, 1024 cells 39 / 35 / 31, 2048 cells 49 / 39 / 37, 4864

@@ -24,16 +24,17 @@ def _built():
 def _cells(where):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     return {"1": 1, "8": 8, "9": 9, "1 part": 8 * sms, "4 lanes": 16 * sms, "2 lanes": 16 * sms + 1,
-            "two waves": 40 * sms - 3, "few terms": 96 * sms, "fused": 96 * sms + 1}[where]
+            "two waves": 40 * sms - 3, "passes": 52 * sms, "few terms": 96 * sms, "fused": 96 * sms + 1}[where]
 
 
 SHAPES = {"200x96": (200, 32, ("silicate", "graphite", "pah")), "37x5": (37, 5, ("silicate",)),
-          "2x1": (2, 1, ("graphite",)), "61x240": (61, 120, ("silicate", "graphite"))}
+          "2x1": (2, 1, ("graphite",)), "61x240": (61, 120, ("silicate", "graphite")),
+          "500x240": (500, 80, ("silicate", "graphite", "pah"))}  # several parts for the weights, ordered cells
 
 
 @pytest.mark.parametrize("form", ["general", "mass", "resid only"])
 @pytest.mark.parametrize("shape", SHAPES)
-@pytest.mark.parametrize("where", ["1", "8", "9", "1 part", "4 lanes", "2 lanes", "two waves", "few terms", "fused"])
+@pytest.mark.parametrize("where", ["1", "8", "9", "1 part", "4 lanes", "2 lanes", "two waves", "passes", "few terms", "fused"])
 def test_split_calls_equal_two_kernel_path(where, shape, form):
     from paper_0907_3768_gb300 import Context, padded_rows
 
