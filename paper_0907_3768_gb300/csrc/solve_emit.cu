@@ -1,8 +1,9 @@
 // Kernel (b): equilibrium-temperature solve and emission SED.  For one
 // request whose emission weights fit in shared memory (dust_solve's usual
-// case) they run as one warp-specialized kernel, k_solve_emit; otherwise, and
-// for the server's work lists of many requests, as two kernels, k_solve and
-// k_emit.  All three give the same bits.
+// case) they run as one warp-specialized kernel, k_solve_emit, or in small
+// calls k_solve_emit_split; otherwise, and for the server's work lists of many
+// requests, as two kernels, k_solve and k_emit.  A large call that stops at
+// the temperatures runs k_solve_grains.  All give the same bits.
 //
 // k_solve — one warp per cell, many warps per SM (the solve is a chain of
 // dependent table lookups, so it wants parallelism, not shared memory):
@@ -53,6 +54,8 @@ constexpr int NB_MAX = 4;     // grains per lane per pass in the solve, at most
 // temperature-only solve: CTAs of SOLVE_TH per SM (measured best: 8 at up to 3 grains per
 // lane, 6 at 4)
 constexpr int solve_tonly_ctas(int nb) { return nb >= 4 ? 6 : 8; }
+// k_solve_grains: threads of its one CTA per SM, grains per group, cells per lane and step
+constexpr int SG_TH = 1024, SG_GL = 16, SG_NB = 2;
 
 // Energy-balance residual emitted / (4 pi absorbed) - 1 of a cell, with
 // emitted = (h + l) 2^(m_c + Ew) and absorbed = (ah + al) 2^(m_c + Eg), all in
@@ -249,6 +252,82 @@ __global__ void __launch_bounds__(SOLVE_TH, TONLY ? solve_tonly_ctas(NB) : (NB >
 #pragma unroll
         for (int i = 0; i < NB; ++i) { s0[i] = s1[i]; n0[i] = n1[i]; }
     }
+}
+
+// The temperature-only solve of a large request, one CTA per SM that stays
+// with SG_GL grains: k_solve has every SM read every grain's table (64 KB each
+// at 4096 nodes), so two of three table loads left its L1 (hit rate 33 %, the
+// path to L2 73 % busy), while 16 grains' visited parts fit there; a lane's
+// grain constants stay in registers as well.  A load takes 64 bytes of two
+// cells' S, whose other grains the CTAs of the other groups read at about the
+// same time, from L2: with 8 grains (32 bytes) 262144 x 96 took the same time
+// but 131072 x 240 264 us for the whole call against 238, with 4 a warp's
+// stores fill half a sector each, and groups one after another in time, not
+// side by side, cost 13 us more.  Solve of 262144 x 96 cells: 126 -> 95 us;
+// what is left is the wavefronts of the scattered table loads.
+// The SMs are whole rounds of the groups and a rest; the rest takes its share
+// of the cells, the last ones, group after group.
+__global__ void __launch_bounds__(SG_TH, 1) k_solve_grains(const __grid_constant__ EmitReq q) {
+    after_previous_kernel();
+    const DevTables &tb = q.tb;
+    const int G = tb.G, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int GL = SG_GL, NB = SG_NB, CL = 32 / GL;    // CL cells per load, NB loads per step
+    constexpr int64_t CTA_CELLS = (SG_TH / 32) * CL * NB;  // cells per step of a CTA
+    const int ng = (G + GL - 1) / GL, b = (int)blockIdx.x, n = (int)gridDim.x;
+    const int slots = n / ng, whole = slots * ng, rest = n - whole;
+    const int64_t head = q.C * whole / n, tail = q.C - head;  // cells of the whole rounds, and of the rest
+    // a whole round's CTA has one group's cells [0, head), every slots-th step;
+    // one of the rest a share [p0, p1) of the tail's cells group after group
+    int64_t p0 = 0, p1 = 0;
+    if (b >= whole) {
+        p0 = tail * ng * (b - whole) / rest;
+        p1 = tail * ng * (b - whole + 1) / rest;
+    }
+    do {
+        int grp = b % ng;
+        int64_t c = b / ng * CTA_CELLS, end = head, step = slots * CTA_CELLS;
+        if (b >= whole) {
+            if (p0 >= p1) break;
+            grp = (int)(p0 / tail);
+            c = head + p0 - grp * tail;
+            end = head + min(tail, p1 - grp * tail);
+            step = CTA_CELLS;
+            p0 = (grp + 1) * tail;
+        }
+        const int g = grp * GL + lane % GL;
+        const bool gok = g < G;
+        const int gc = gok ? g : 0;
+        const float4 gq1 = __ldg(reinterpret_cast<const float4 *>(tb.gp) + gc);
+        const float *S = q.S + gc;
+        c += warp * CL * NB + lane / GL;
+        float s[NB];
+#pragma unroll
+        for (int i = 0; i < NB; ++i) s[i] = c + CL * i < end ? __ldg(S + (c + CL * i) * tb.Gs) : 0.f;
+        for (; c - lane / GL < end; c += step) {
+            // the next step's loads ahead of this one's lookups
+            float sn[NB];
+#pragma unroll
+            for (int i = 0; i < NB; ++i) {
+                const int64_t cell = c + step + CL * i;
+                sn[i] = cell < end ? __ldg(S + cell * tb.Gs) : 0.f;
+            }
+            int gi[NB], fl[NB];
+            float4 gq[NB];
+            float T[NB];
+#pragma unroll
+            for (int i = 0; i < NB; ++i) { gi[i] = gc; gq[i] = gq1; }
+            solve_batch<NB>(tb, gi, s, gq, T, fl);
+#pragma unroll
+            for (int i = 0; i < NB; ++i) {
+                const int64_t cell = c + CL * i;
+                if (gok && cell < end) {
+                    q.T[cell * G + g] = T[i];
+                    if (q.flags) q.flags[cell * G + g] = (uint8_t)fl[i];
+                }
+                s[i] = sn[i];
+            }
+        }
+    } while (b >= whole);
 }
 
 // One grain's term for two wavelengths of one cell, folded into the group's
@@ -1100,7 +1179,16 @@ int launch_emit_batch(EmitBatch &B, int num_sms, cudaStream_t st, cudaEvent_t be
         const int64_t grid = std::min<int64_t>((cells * 32 + SOLVE_TH - 1) / SOLVE_TH, (int64_t)num_sms * 16);
         bool tonly = true;
         for (int i = 0; i < B.nreq; ++i) tonly = tonly && !(B.req[i].mode & EMIT_ON);
-        if (tonly) {
+        // One request of many cells stops at T: a CTA per SM stays with a few
+        // grains.  Below 128 cells per SM the many small CTAs of k_solve fill
+        // the SMs better (whole calls, k_solve first: 96 grains 16384 cells
+        // 26.2 us against 27.6, 32768 41.0 against 40.4, 131072 104 against
+        // 89; 240 grains 8192 35 against 37, 32768 88 against 82, 131072 294
+        // against 238; 12 grains 131072 64 against 44).
+        const int groups = (B.req[0].tb.G + SG_GL - 1) / SG_GL;
+        if (tonly && B.nreq == 1 && cells > (int64_t)128 * num_sms && groups <= num_sms) {
+            DUST_CUDA_TRY(launch_early(early, k_solve_grains, (unsigned)num_sms, SG_TH, 0, st, B.req[0]));
+        } else if (tonly) {
             switch (nb) {
                 case 1: DUST_CUDA_TRY(launch_early(early, k_solve<1, true>, (unsigned)grid, SOLVE_TH, 0, st, B)); break;
                 case 2: DUST_CUDA_TRY(launch_early(early, k_solve<2, true>, (unsigned)grid, SOLVE_TH, 0, st, B)); break;
