@@ -27,7 +27,13 @@ namespace dust {
 namespace {
 
 constexpr int ORD_TH = 256;            // threads per CTA
-constexpr int ORD_CPB = ORD_TH * 8;    // cells per CTA
+// Cells per thread, all of their loads in flight at once and their classes
+// kept in registers (the kernels are chains of global latencies: 20011 x 200 x
+// 96, the whole solve 111.8 us with a loop of loads, 111.1 so).  With 4 cells
+// 109.7 but 262144 cells 919 us against 917; with 2 or 1, 117: smaller CTAs
+// mix the cells of a class more, and a tile's rows lie further apart.
+constexpr int ORD_CPT = 8;
+constexpr int ORD_CPB = ORD_TH * ORD_CPT;  // cells per CTA
 
 __device__ __forceinline__ int key_class(float v) {
     return v > 0.f ? min(__float_as_int(v) >> 21, NBK - 1) : 0;
@@ -57,8 +63,17 @@ __global__ void __launch_bounds__(ORD_TH) k_order_classify(const __grid_constant
     let_next_kernel_start();
     after_previous_kernel();
     __syncthreads();
-    for (int64_t c = c0 + threadIdx.x; c < c1; c += ORD_TH) {
-        const int b = key_class(__ldg(q.key + c * q.kstride));
+    float key[ORD_CPT];  // all of them in flight at once
+#pragma unroll
+    for (int j = 0; j < ORD_CPT; ++j) {
+        const int64_t c = c0 + threadIdx.x + j * ORD_TH;
+        key[j] = c < c1 ? __ldg(q.key + c * q.kstride) : 0.f;
+    }
+#pragma unroll
+    for (int j = 0; j < ORD_CPT; ++j) {
+        const int64_t c = c0 + threadIdx.x + j * ORD_TH;
+        if (c >= c1) break;
+        const int b = key_class(key[j]);
         q.bkt[c] = (uint16_t)b;
         atomicAdd(&cnt[b], 1u);
     }
@@ -77,8 +92,15 @@ __global__ void __launch_bounds__(ORD_TH) k_order_scatter(const __grid_constant_
     const int64_t c0 = (int64_t)(blockIdx.x - q.block_begin) * ORD_CPB;
     const int64_t c1 = min(c0 + ORD_CPB, q.C);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int i = tid; i < NBK; i += ORD_TH) cnt[i] = 0u;
     let_next_kernel_start();
     after_previous_kernel();
+    int b[ORD_CPT];  // this thread's cells' classes, on their way during the scan
+#pragma unroll
+    for (int j = 0; j < ORD_CPT; ++j) {
+        const int64_t c = c0 + tid + j * ORD_TH;
+        b[j] = c < c1 ? q.bkt[c] : -1;
+    }
     // exclusive scan of the NBK counts: four consecutive classes per thread
     constexpr int PER = NBK / ORD_TH;
     unsigned v[PER], s = 0;
@@ -91,26 +113,24 @@ __global__ void __launch_bounds__(ORD_TH) k_order_scatter(const __grid_constant_
         if (lane >= o) inc += y;
     }
     if (lane == 31) wsum[warp] = inc;
-    for (int i = tid; i < NBK; i += ORD_TH) cnt[i] = 0u;
     __syncthreads();
     unsigned off = 0;
     for (int w = 0; w < warp; ++w) off += wsum[w];
     unsigned run = off + inc - s;
 #pragma unroll
     for (int j = 0; j < PER; ++j) { base[tid * PER + j] = run; run += v[j]; }
-    // this CTA's count per class
-    for (int64_t c = c0 + tid; c < c1; c += ORD_TH) atomicAdd(&cnt[q.bkt[c]], 1u);
+    // this CTA's count per class, and each cell's place in it
+    unsigned place[ORD_CPT];
+#pragma unroll
+    for (int j = 0; j < ORD_CPT; ++j) place[j] = b[j] >= 0 ? atomicAdd(&cnt[b[j]], 1u) : 0u;
     __syncthreads();
     // reserve: base becomes this CTA's first slot of each class
-    for (int i = tid; i < NBK; i += ORD_TH) {
+    for (int i = tid; i < NBK; i += ORD_TH)
         if (cnt[i]) base[i] += atomicAdd(q.hist + NBK + i, cnt[i]);
-        cnt[i] = 0u;
-    }
     __syncthreads();
-    for (int64_t c = c0 + tid; c < c1; c += ORD_TH) {
-        const int b = q.bkt[c];
-        q.order[base[b] + atomicAdd(&cnt[b], 1u)] = (int)c;
-    }
+#pragma unroll
+    for (int j = 0; j < ORD_CPT; ++j)
+        if (b[j] >= 0) q.order[base[b[j]] + place[j]] = (int)(c0 + tid + j * ORD_TH);
 }
 
 }  // namespace
