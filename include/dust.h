@@ -343,8 +343,10 @@ int dust_solve_mass(dust_ctx *ctx, int64_t n_cells, const float *J, int64_t ld, 
  *                      solve.  L is required.
  *  *iters_done         solves run; *last_change the last measured change
  *                      (infinite until two solves have run).  Either may be NULL.
- * Synchronises `stream` once per iteration (the stop test is read on the
- * host).  The context keeps a working J and the previous L (8 C ld bytes). */
+ * Waits on the host once per iteration from the second on (the stop test is
+ * read there; the next solve's absorption may run meanwhile) and returns with
+ * nothing of its own left in `stream`.  The context keeps a working J and the
+ * previous L (8 C ld bytes). */
 int dust_solve_coupled(dust_ctx *ctx, int64_t n_cells, const float *J_ext, int64_t ld, const float *E,
                        const float *n, int max_iters, double tol, float *T, float *L, double *resid,
                        uint8_t *flags, int *iters_done, double *last_change, void *stream);

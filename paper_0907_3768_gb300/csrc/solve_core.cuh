@@ -1,8 +1,8 @@
-// Device arithmetic shared by the two temperature-solve kernels (the
-// stand-alone solve and the absorption GEMM whose epilogue solves): MUFU
-// wrappers, float-float accumulation and the table root solve of Eq. 7.
-// Both kernels take every result through these functions, so they agree
-// bit for bit.
+// Device arithmetic shared by the temperature-solve kernels (the stand-alone
+// ones, those that emit as well, and the absorption GEMM whose epilogue
+// solves): MUFU wrappers, float-float accumulation and the table root solve of
+// Eq. 7.  All take every result through these functions, so they agree bit for
+// bit.
 #pragma once
 
 #include "dust_internal.cuh"

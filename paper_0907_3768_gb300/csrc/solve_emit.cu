@@ -577,7 +577,7 @@ __device__ __forceinline__ void emit_item_out(const EmitReq &q, int64_t cell, in
 // the previous pass left in the scratch (accp) and the last one finishes
 // them, so every item adds its groups in the same order as one pass would.
 // Per CTA one copier warp fills KE_NBUF pair-tile buffers from the scratch
-// (cp.async, 8 bytes per pair) and KE_W emission warps claim the items in
+// (cp.async, 8 bytes per pair) and ke_warps emission warps claim the items in
 // order (one k-group of one tile, its cells on the 32 lanes, emit_item), the
 // longest wavelengths of a tile first.  Hand-over through monotone counters
 // per buffer: the copier adds 1 to filled[b] per tile, emission warps add 1
@@ -585,8 +585,18 @@ __device__ __forceinline__ void emit_item_out(const EmitReq &q, int64_t cell, in
 // emitted once filled[b] >= i / KE_NBUF + 1, and refilled once drained[b]
 // counts every item of the tiles put there before it.  Waits poll with a
 // short sleep, are bounded, and record DUST_ETIMEOUT.
-constexpr int KE_W = 23;                // emission warps (15 of 128 registers: 3 % slower)
-constexpr int KE_TH = (KE_W + 1) * 32;  // and one copier warp: 768 threads, 80 registers
+// Emission warps: 15 that claim an item when they begin it (with the copier
+// 512 threads of 128 registers); with MANY 23 that claim the next one while
+// they emit one (768 threads of 80).  MANY needs tiles of at least as many
+// items as its warps hold, 46: with fewer, items claimed and not yet begun
+// keep the three buffers from being refilled.  Whole solves in two kernels, 15
+// and 23: 200 x 96 (25 items) 262144 cells 1.20 and 1.60 ms, 350 x 96 (44)
+// 65536 cells 0.530 and 0.544, 500 x 240 (63) 65536 cells 1.718 and 1.694;
+// 131072 cells 500 x 240, of which these are the later grain passes, 3.03 and
+// 2.94 ms.
+constexpr int KE_MANY = 23;
+constexpr int ke_warps(bool many) { return many ? KE_MANY : 15; }
+constexpr int ke_th(bool many) { return (ke_warps(many) + 1) * 32; }
 constexpr int KE_NBUF = 3;
 
 __device__ __forceinline__ void cp_async8(void *dst, const void *src) {
@@ -634,8 +644,8 @@ __device__ __forceinline__ bool warp_wait_geq(const int *ctr, int target, volati
     return ok != 0;
 }
 
-template <bool MASS>
-__global__ void __launch_bounds__(KE_TH, 1) k_emit(const __grid_constant__ EmitBatch B) {
+template <bool MASS, bool MANY>
+__global__ void __launch_bounds__(ke_th(MANY), 1) k_emit(const __grid_constant__ EmitBatch B) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int TC = KE_TC;
     constexpr int PW = MASS ? 1 : 2;  // floats per pair
@@ -657,7 +667,7 @@ __global__ void __launch_bounds__(KE_TH, 1) k_emit(const __grid_constant__ EmitB
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     {
         const float4 *src = reinterpret_cast<const float4 *>(tb.Chat);
-        for (int i = tid; i < NKG * 2 * gc; i += KE_TH) {
+        for (int i = tid; i < NKG * 2 * gc; i += ke_th(MANY)) {
             const int kg = i / (2 * gc), o = i - kg * 2 * gc;
             sC[(size_t)kg * CST + o] = __ldg(src + ((size_t)kg * G8 + q.g0) * 2 + o);
         }
@@ -667,7 +677,7 @@ __global__ void __launch_bounds__(KE_TH, 1) k_emit(const __grid_constant__ EmitB
     __syncthreads();
     if (ntl <= 0) return;
 
-    if (warp == KE_W) {
+    if (warp == ke_warps(MANY)) {
         // ------------------------------------------------------------ copier
         int expect[KE_NBUF] = {};  // items of the tiles put in each buffer so far
         for (int i = 0; i < ntl; ++i) {
@@ -697,17 +707,24 @@ __global__ void __launch_bounds__(KE_TH, 1) k_emit(const __grid_constant__ EmitB
         const bool rs = (q.mode & EMIT_RESID) != 0, storeL = (q.mode & EMIT_STORE_L) != 0;
         const bool vecL = storeL && ((reinterpret_cast<uintptr_t>(q.L) & 15) == 0) && (q.ld % 4 == 0);
         int i = 0, rem = 0;  // the claimed item: tile of the unit, item in it
-        {
-            int w = 0;
-            if (lane == 0) w = atomicAdd(claim, 1);
-            rem = __shfl_sync(0xffffffffu, w, 0);
+        if (MANY) {
+            if (lane == 0) rem = atomicAdd(claim, 1);
+            rem = __shfl_sync(0xffffffffu, rem, 0);
         }
         for (;;) {
-            for (; rem >= NKG; rem -= NKG) ++i;
-            if (i >= ntl) break;
-            // the next item is claimed now, so that the counter's latency hides behind this one
             int w = 0;
-            if (lane == 0) w = atomicAdd(claim, 1);
+            if (MANY) {
+                for (; rem >= NKG; rem -= NKG) ++i;
+                if (i >= ntl) break;
+                // the next item is claimed now, so that the counter's latency hides behind this one
+                if (lane == 0) w = atomicAdd(claim, 1);
+            } else {
+                if (lane == 0) w = atomicAdd(claim, 1);
+                w = __shfl_sync(0xffffffffu, w, 0);
+                i = w / NKG;
+                if (i >= ntl) break;
+                rem = w - i * NKG;
+            }
             const int ikg = NKG - 1 - rem;
             const int b = i % KE_NBUF;
             if (!warp_wait_geq(&filled[b], i / KE_NBUF + 1, abort_flag, tb.status, lane)) break;
@@ -734,21 +751,25 @@ __global__ void __launch_bounds__(KE_TH, 1) k_emit(const __grid_constant__ EmitB
             }
             __syncwarp();
             if (lane == 0) add_release_cta(&drained[b], 1);
-            rem = __shfl_sync(0xffffffffu, w, 0) - i * NKG;
+            if (MANY) rem = __shfl_sync(0xffffffffu, w, 0) - i * NKG;
         }
     }
 }
 
 // Residual of one cell (Eq. 6 against Eqs. 8-10, see residual()) from its
 // k-group partials, summed in ascending order, and its cell record.
+// SAME: they may come from another SM in the same kernel, so they are read
+// through L2.  (After the emission kernel L1 may hold the lines of a row from
+// one partial to the next: 262144 cells in two kernels 1.196 ms without, 1.188
+// with it.)
+template <bool SAME = true>
 __device__ __forceinline__ void cell_resid(const EmitReq &q, int64_t cell) {
     const int NKG = q.tb.NKG;
     const float2 *pp = q.part + cell * NKG;
     float h = 0.f, l = 0.f;
-    // through L2: the partials may be another SM's
 #pragma unroll 8
     for (int kg = 0; kg < NKG; ++kg) {
-        const float2 v = __ldcg(pp + kg);
+        const float2 v = SAME ? __ldcg(pp + kg) : pp[kg];
         ff_add(h, l, v.x, v.y);
     }
     const int4 cv = __ldcg(reinterpret_cast<const int4 *>(q.cell + cell));
@@ -1059,7 +1080,7 @@ __global__ void __launch_bounds__(SOLVE_TH) k_resid(const __grid_constant__ Emit
         while (ri + 1 < E.nreq && u >= E.req[ri + 1].cell_begin) ++ri;
         const EmitReq &q = E.req[ri];
         if (!(q.mode & EMIT_RESID)) continue;
-        cell_resid(q, u - q.cell_begin);
+        cell_resid<false>(q, u - q.cell_begin);
     }
 }
 
@@ -1231,10 +1252,12 @@ int launch_emit_batch(EmitBatch &B, int num_sms, cudaStream_t st, cudaEvent_t be
                 units += ((E.req[k].C + KE_TC - 1) / KE_TC + tpu - 1) / tpu;
             }
             E.ntiles = tiles;
-            const void *kern = mass ? reinterpret_cast<const void *>(k_emit<true>) : reinterpret_cast<const void *>(k_emit<false>);
+            bool many = true;  // every request's tiles have the items that 23 warps hold
+            for (int k = 0; k < E.nreq; ++k) many = many && E.req[k].tb.NKG >= 2 * KE_MANY;
+            auto kern = mass ? (many ? k_emit<true, true> : k_emit<true, false>)
+                             : (many ? k_emit<false, true> : k_emit<false, false>);
             DUST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            if (mass) k_emit<true><<<(unsigned)units, KE_TH, smem, st>>>(E);
-            else k_emit<false><<<(unsigned)units, KE_TH, smem, st>>>(E);
+            kern<<<(unsigned)units, ke_th(many), smem, st>>>(E);
             DUST_CUDA_TRY(cudaGetLastError());
             ++nl;
             E.nreq = 0;
