@@ -41,10 +41,10 @@ KERNEL_SOURCES = {
 }
 RECORDED_TRAFFIC = {
     # kernel: (bytes per launch on the bench's workload, profile summary, sources sha256[:16])
-    "k_solve_emit": (234.642176e6 + 358.232064e6, "profiles/k_solve_emit_2e18cells_K200_G96.md", "1b2b671c702a6864"),
-    "k_emit": (220.631808e6 + 218.775808e6, "profiles/k_emit_2e18cells_K200_G96.md", "1b2b671c702a6864"),
+    "k_solve_emit": (248.616192e6 + 361.798144e6, "profiles/k_solve_emit_2e18cells_K200_G96.md", "e3f7ff69c06fdd0b"),
+    "k_emit": (220.736256e6 + 218.525952e6, "profiles/k_emit_2e18cells_K200_G96.md", "e3f7ff69c06fdd0b"),
     # the full-size launch, DRAM counters only (one ncu pass; the 2^14-cell --set full capture is in the same file)
-    "k_fluct": (255.956992e6 + 175.320064e6, "profiles/k_fluct_2e14cells_K200_G36_M128.md", "2eac562135043b6a"),
+    "k_fluct": (255.166208e6 + 175.692800e6, "profiles/k_fluct_2e14cells_K200_G36_M128.md", "b3d8c7bb4178b4a4"),
 }
 
 

@@ -256,15 +256,16 @@ __global__ void __launch_bounds__(SOLVE_TH, TONLY ? solve_tonly_ctas(NB) : (NB >
 
 // The temperature-only solve of a large request, one CTA per SM that stays
 // with SG_GL grains: k_solve has every SM read every grain's table (64 KB each
-// at 4096 nodes), so two of three table loads left its L1 (hit rate 33 %, the
-// path to L2 73 % busy), while 16 grains' visited parts fit there; a lane's
-// grain constants stay in registers as well.  A load takes 64 bytes of two
+// at 4096 nodes), so nearly every table load left its L1 (3 % hits), and it
+// loads the grain's constants anew for every cell.  With 16 grains the tables'
+// visited parts stay in L1 in part (30 % hits) and the constants in registers:
+// 28 M sectors loaded instead of 41 M.  A load takes 64 bytes of two
 // cells' S, whose other grains the CTAs of the other groups read at about the
 // same time, from L2: with 8 grains (32 bytes) 262144 x 96 took the same time
 // but 131072 x 240 264 us for the whole call against 238, with 4 a warp's
 // stores fill half a sector each, and groups one after another in time, not
-// side by side, cost 13 us more.  Solve of 262144 x 96 cells: 126 -> 95 us;
-// what is left is the wavefronts of the scattered table loads.
+// side by side, cost 13 us more.  Solve of 262144 x 96 cells: 126 -> 95 us,
+// bound by L1's requests to L2 (79 % of their peak over the kernel).
 // The SMs are whole rounds of the groups and a rest; the rest takes its share
 // of the cells, the last ones, group after group.
 __global__ void __launch_bounds__(SG_TH, 1) k_solve_grains(const __grid_constant__ EmitReq q) {
