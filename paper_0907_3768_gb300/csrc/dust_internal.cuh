@@ -311,6 +311,10 @@ const char *cuda_err_name(cudaError_t e);
 // kernel before it lets it start with let_next_kernel_start().  Every CTA of
 // both has to pass after_previous_kernel() when it was itself launched so, so
 // that its end implies the end of what came before.  (early = false: a plain launch.)
+// What an earlier kernel of the call writes (S, the order, the pairs and
+// records) is read by plain loads: it changes during the early kernel's life, so
+// it is no read-only data, and a load through that path (__ldg) need not stay
+// behind the wait.
 // An SM keeps its split of L1 and shared memory while CTAs are on it, so a
 // kernel that starts beside the tensor-core GEMM runs with the 28 KB of L1 that
 // its rings leave; the solves want more (262144 x 200 x 96: 919 us per step

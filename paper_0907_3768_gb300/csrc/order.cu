@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(ORD_TH) k_order_classify(const __grid_constant
 #pragma unroll
     for (int j = 0; j < ORD_CPT; ++j) {
         const int64_t c = c0 + threadIdx.x + j * ORD_TH;
-        key[j] = c < c1 ? __ldg(q.key + c * q.kstride) : 0.f;
+        key[j] = c < c1 ? q.key[c * q.kstride] : 0.f;
     }
 #pragma unroll
     for (int j = 0; j < ORD_CPT; ++j) {

@@ -88,7 +88,7 @@ __device__ __forceinline__ void load_pass(const EmitReq &q, int64_t cell, int gb
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
         const int g = gb + lane + 32 * i;
-        s[i] = g < G ? __ldg(Srow + g) : 0.f;
+        s[i] = g < G ? Srow[g] : 0.f;
         nv[i] = (with_n && g < G) ? __ldg(nrow + g) : 0.f;
     }
 }
@@ -303,14 +303,14 @@ __global__ void __launch_bounds__(SG_TH, 1) k_solve_grains(const __grid_constant
         c += warp * CL * NB + lane / GL;
         float s[NB];
 #pragma unroll
-        for (int i = 0; i < NB; ++i) s[i] = c + CL * i < end ? __ldg(S + (c + CL * i) * tb.Gs) : 0.f;
+        for (int i = 0; i < NB; ++i) s[i] = c + CL * i < end ? S[(c + CL * i) * tb.Gs] : 0.f;
         for (; c - lane / GL < end; c += step) {
             // the next step's loads ahead of this one's lookups
             float sn[NB];
 #pragma unroll
             for (int i = 0; i < NB; ++i) {
                 const int64_t cell = c + step + CL * i;
-                sn[i] = cell < end ? __ldg(S + cell * tb.Gs) : 0.f;
+                sn[i] = cell < end ? S[cell * tb.Gs] : 0.f;
             }
             int gi[NB], fl[NB];
             float4 gq[NB];
@@ -513,7 +513,7 @@ __device__ __forceinline__ float load_nax(const DevTables &tb, int ikg, float2 (
 
 // Cell of slot i of a request's emission order.
 __device__ __forceinline__ int64_t ordered_cell(const EmitReq &q, int64_t i) {
-    return q.order ? (int64_t)__ldg(q.order + i) : i;
+    return q.order ? (int64_t)q.order[i] : i;
 }
 
 
