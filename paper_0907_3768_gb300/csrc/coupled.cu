@@ -28,6 +28,7 @@ constexpr int CPL_TH = 128;
 // lane), and L stays in registers between its two uses.  16384 x 200 out of memory:
 // 24 -> 19 us (79 MB: 12 us at the copy rate).
 constexpr int CPL_V = 2;
+constexpr unsigned int NOT_YET = 0x7f800000u;  // infinity: the host's word where no change has been measured
 
 template <bool VEC>
 __global__ void __launch_bounds__(CPL_TH) k_couple(int64_t C, int K, int64_t ld, const float *Jext,
@@ -96,7 +97,8 @@ __global__ void __launch_bounds__(CPL_TH) k_couple(int64_t C, int K, int64_t ld,
         __threadfence();
         if (atomicAdd(count, 1u) == gridDim.x - 1) {
             __threadfence();
-            *host = atomicExch(change, 0u);
+            const unsigned int c = atomicExch(change, 0u);
+            *host = first ? NOT_YET : c;
             *count = 0u;
             __threadfence_system();
         }
@@ -159,8 +161,9 @@ extern "C" int dust_solve_coupled(dust_ctx *ctx, int64_t n_cells, const float *J
             ctx->cpl_bytes = 0;
             e = cudaMalloc(&ctx->cpl, need);
         }
-        // columns K..ld of the working J are read as padding by nothing, but keep them defined
-        if (e == cudaSuccess) e = cudaMemset(ctx->cpl, 0, need);
+        // columns K..ld of the working J are read as padding by nothing, but keep them defined;
+        // cleared in `st`, since nothing orders another stream's clear before the passes
+        if (e == cudaSuccess) e = cudaMemsetAsync(ctx->cpl, 0, need, st);
         if (e == cudaSuccess) ctx->cpl_bytes = need;
         else rc = set_error(DUST_ENOMEM, "coupled-solve buffers: %s", cudaGetErrorString(e));
     }
@@ -204,6 +207,9 @@ extern "C" int dust_solve_coupled(dust_ctx *ctx, int64_t n_cells, const float *J
         absorbed = false;
         if (rc != DUST_OK) break;
         ++it;
+        // a pass that left no change must not pass for one that left a small one
+        // (the first one's word, not waited for, says the same)
+        *(volatile unsigned int *)ctx->cpl_host = NOT_YET;
         cudaError_t e = launch_early(true, vec ? k_couple<true> : k_couple<false>, (unsigned)grid, CPL_TH, 0, st, n_cells, ctx->K, ld,
                                      J_ext, E, (const float *)L, Lprev, Jw, (int)(it == 1), chg, chg + 1,
                                      (volatile unsigned int *)ctx->cpl_host);
