@@ -1066,6 +1066,7 @@ __global__ void __launch_bounds__(SPL_TH, 2) k_solve_emit_split(const __grid_con
             __threadfence();
         }
         last = __shfl_sync(0xffffffffu, last, 0);
+        __syncwarp();  // the shuffle orders no memory: this puts every lane's reads after lane 0's count
     }
     if (last && lane < nc) cell_resid(q, ordered_cell(q, c0 + lane));
 }
