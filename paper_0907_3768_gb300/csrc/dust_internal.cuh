@@ -305,6 +305,21 @@ const char *cuda_err_name(cudaError_t e);
         }                                                                            \
     } while (0)
 
+// Lets a kernel be launched with as much dynamic shared memory as the device
+// gives.  The limit belongs to the function, for every thread and context of the
+// process, so it is never set to one call's own need: another call's smaller need
+// between this one's setting and its launch would have the launch refused.  (For
+// kernels without static shared memory, which would count against the limit; a
+// launch still takes only the bytes it names.)
+template <class Kernel>
+cudaError_t allow_shared_memory(Kernel *kernel) {
+    int dev = 0, most = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    return e;
+}
+
 // Launch of a kernel that may start while the kernel before it in the stream
 // still runs: its CTAs take their places and read what only the context holds,
 // then wait in after_previous_kernel() for that kernel's end and writes.  The

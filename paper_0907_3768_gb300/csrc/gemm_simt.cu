@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(NTH, TN <= 6 ? 3 : 2) k_gemm_simt(const __grid
 template <int TN>
 int launch_simt(const SimtBatch &B, unsigned grid, cudaStream_t st) {
     constexpr int smem = NST * stage_floats(TN) * (int)sizeof(float);
-    DUST_CUDA_TRY(cudaFuncSetAttribute(k_gemm_simt<TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    DUST_CUDA_TRY(allow_shared_memory(k_gemm_simt<TN>));
     k_gemm_simt<TN><<<grid, NTH, smem, st>>>(B);
     DUST_CUDA_TRY(cudaGetLastError());
     return DUST_OK;

@@ -905,11 +905,11 @@ template <bool BF16, bool TWO_PASS>
 int launch_t(const TcBatch &B, size_t smem, int grid, cudaStream_t st, const SolveList *sl) {
     if (B.orient == 1) {
         auto kern = B.bn == BN_T ? k_gemm_tc_t<BF16, TWO_PASS, BN_T> : k_gemm_tc_t<BF16, TWO_PASS, BN_S>;
-        DUST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        DUST_CUDA_TRY(allow_shared_memory(kern));
         kern<<<grid, NTHREADS_T, smem, st>>>(B);
     } else if (sl) {
         auto kern = k_absorb_solve<BF16, TWO_PASS>;
-        DUST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        DUST_CUDA_TRY(allow_shared_memory(kern));
         // the smallest shared-memory carveout that holds the rings: the rest is L1
         const int pct = (int)std::min<size_t>(100, (smem + 2048) * 100 / (228 * 1024) + 1);
         DUST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, pct));
@@ -918,7 +918,7 @@ int launch_t(const TcBatch &B, size_t smem, int grid, cudaStream_t st, const Sol
         kern<<<grid, block, smem, st>>>(B, *sl);
     } else {
         auto kern = k_gemm_tc<BF16, TWO_PASS>;
-        DUST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        DUST_CUDA_TRY(allow_shared_memory(kern));
         kern<<<grid, NTHREADS, smem, st>>>(B);
     }
     DUST_CUDA_TRY(cudaGetLastError());

@@ -1258,7 +1258,7 @@ int launch_emit_batch(EmitBatch &B, int num_sms, cudaStream_t st, cudaEvent_t be
             for (int k = 0; k < E.nreq; ++k) many = many && E.req[k].tb.NKG >= 2 * KE_MANY;
             auto kern = mass ? (many ? k_emit<true, true> : k_emit<true, false>)
                              : (many ? k_emit<false, true> : k_emit<false, false>);
-            DUST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            DUST_CUDA_TRY(allow_shared_memory(kern));
             kern<<<(unsigned)units, ke_th(many), smem, st>>>(E);
             DUST_CUDA_TRY(cudaGetLastError());
             ++nl;
@@ -1355,7 +1355,7 @@ int launch_fse(const EmitReq &r, int nb, unsigned grid, size_t smem, bool early,
                      : nb == 2 ? reinterpret_cast<const void *>(k_solve_emit<2, MASS, PASS>)
                      : nb == 3 ? reinterpret_cast<const void *>(k_solve_emit<3, MASS, PASS>)
                                : reinterpret_cast<const void *>(k_solve_emit<4, MASS, PASS>);
-    DUST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    DUST_CUDA_TRY(allow_shared_memory(kern));
     switch (nb) {
         case 1: DUST_CUDA_TRY(launch_early(early, k_solve_emit<1, MASS, PASS>, grid, fse_th(PASS), smem, st, r)); break;
         case 2: DUST_CUDA_TRY(launch_early(early, k_solve_emit<2, MASS, PASS>, grid, fse_th(PASS), smem, st, r)); break;
@@ -1409,7 +1409,7 @@ template <bool MASS, int LPC>
 int launch_split(const EmitReq &r, int nb, unsigned grid, const SplitPlan &p, int *cnt, cudaStream_t st) {
     auto kern = nb == 1 ? k_solve_emit_split<1, MASS, LPC> : nb == 2 ? k_solve_emit_split<2, MASS, LPC>
               : nb == 3 ? k_solve_emit_split<3, MASS, LPC> : k_solve_emit_split<4, MASS, LPC>;
-    DUST_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem));
+    DUST_CUDA_TRY(allow_shared_memory(kern));
     DUST_CUDA_TRY(launch_early(true, kern, grid, SPL_TH, p.smem, st, r, p.parts, cnt));
     return DUST_OK;
 }
