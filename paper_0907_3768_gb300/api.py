@@ -5,6 +5,7 @@ library's kernels.  There is no CPU fallback: without the built library or a
 CUDA device the calls raise.
 """
 import ctypes
+import warnings
 
 import numpy as np
 import torch
@@ -35,6 +36,16 @@ def padded_rows(J, multiple=4):
     return buf[:, :K]
 
 
+def _front_or_none():
+    """The front end's native half, or None with a warning: it shortens a call's host side and computes
+    nothing, so a context needs libdust.so alone."""
+    try:
+        return _lib.front()
+    except (RuntimeError, ImportError, OSError) as e:
+        warnings.warn(f"calls take their host side in Python: {e}", RuntimeWarning, stacklevel=3)
+        return None
+
+
 class Context:
     """One wavelength grid + grain set, with its tables resident on `device`."""
 
@@ -51,7 +62,7 @@ class Context:
                                            int(device))
         self.K, self.G, self.device = K, G, int(device)
         self.T_min, self.T_max = float(T_min), float(T_max)
-        self._front = _lib.front()
+        self._front = _front_or_none()
         self._solve, self._solve_mass = _lib.address("dust_solve"), _lib.address("dust_solve_mass")
 
     @classmethod
@@ -111,11 +122,20 @@ class Context:
         return C, J.stride(0)
 
     def alloc_outputs(self, C, ld, want_L=True, want_resid=True, want_flags=True):
-        return self._front.alloc_outputs(C, self.G, self.K, ld, self.device, want_L, want_resid, want_flags)
+        if self._front is not None:
+            return self._front.alloc_outputs(C, self.G, self.K, ld, self.device, want_L, want_resid, want_flags)
+        dev = torch.device("cuda", self.device)
+        out = dict(T=torch.empty((C, self.G), dtype=torch.float32, device=dev))
+        out["L_buf"] = torch.empty((C, ld), dtype=torch.float32, device=dev) if want_L else None
+        out["L"] = out["L_buf"][:, :self.K] if want_L else None
+        out["resid"] = torch.empty((C,), dtype=torch.float64, device=dev) if want_resid else None
+        out["flags"] = torch.empty((C, self.G), dtype=torch.uint8, device=dev) if want_flags else None
+        return out
 
     def _solve_new(self, fn, J, n, mass, want_L, want_resid, want_flags):
-        """One native call into new outputs on the current stream; None where J or n is not what it takes."""
-        if self.handle is None or not isinstance(J, torch.Tensor) or not isinstance(n, torch.Tensor):
+        """One native call into new outputs on the current stream; None where J or n is not what it takes,
+        or where the native half is missing."""
+        if self._front is None or self.handle is None or not isinstance(J, torch.Tensor) or not isinstance(n, torch.Tensor):
             return None
         r = self._front.solve(fn, self.handle, self.G, self.K, self.device, J, n, mass, bool(want_L), bool(want_resid),
                               bool(want_flags))

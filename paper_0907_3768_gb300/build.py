@@ -12,6 +12,7 @@ import shutil
 import subprocess
 import sys
 import sysconfig
+import warnings
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
@@ -71,11 +72,16 @@ def build_front(force=False):
 
 
 def build(force=False, verbose=False, ptxas_verbose=False):
-    """Compile and link libdust.so and the _front module; returns libdust.so's path."""
+    """Compile and link libdust.so and the _front module; returns libdust.so's path.
+    Where _front cannot be built (no torch headers, another ABI) that is a warning: the Python
+    front end works without it."""
     with cf.ThreadPoolExecutor(max_workers=1) as ex:
         front = ex.submit(build_front, force)
         lib = build_lib(force, verbose, ptxas_verbose)
-        front.result()
+        try:
+            front.result()
+        except (RuntimeError, ImportError, OSError) as e:
+            warnings.warn(f"the front end's native half was not built: {e}", RuntimeWarning, stacklevel=2)
     return lib
 
 
