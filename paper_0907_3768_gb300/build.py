@@ -6,6 +6,7 @@ paper_0907_3768_gb300/_build/libdust.so with the CUDA runtime linked
 statically (the library then needs only the driver at run time).
 """
 import concurrent.futures as cf
+import contextlib
 import glob
 import os
 import shutil
@@ -20,6 +21,7 @@ OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libdust.so")
 FRONT_SRC = os.path.join(CSRC, "front.cpp")
 FRONT = os.path.join(OUT, "_front" + sysconfig.get_config_var("EXT_SUFFIX"))
+FRONT_STAMP = FRONT + ".built_against"
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
@@ -49,15 +51,34 @@ def up_to_date():
     return all(os.path.getmtime(p) <= t for p in _deps())
 
 
+def front_built_against():
+    """What a _front module holds for: the torch whose headers, ABI and libraries it was compiled against."""
+    import torch
+
+    return f"torch {torch.__version__} in {os.path.dirname(torch.__file__)}, C++11 ABI {int(torch._C._GLIBCXX_USE_CXX11_ABI)}\n"
+
+
+def front_up_to_date():
+    if not (os.path.exists(FRONT) and os.path.exists(FRONT_STAMP)):
+        return False
+    t = os.path.getmtime(FRONT)
+    if any(os.path.getmtime(p) > t for p in (FRONT_SRC, os.path.join(INCLUDE, "dust.h"), os.path.abspath(__file__))):
+        return False
+    with open(FRONT_STAMP) as f:
+        return f.read() == front_built_against()
+
+
 def build_front(force=False):
     """Compile and link the _front module; returns its path."""
-    deps = [FRONT_SRC, os.path.join(INCLUDE, "dust.h")]
-    if not force and os.path.exists(FRONT) and all(os.path.getmtime(p) <= os.path.getmtime(FRONT) for p in deps):
+    if not force and front_up_to_date():
         return FRONT
     import torch
     from torch.utils import cpp_extension
 
     os.makedirs(OUT, exist_ok=True)
+    for old in (FRONT_STAMP, FRONT):  # a module of another torch must not stay where this build fails
+        with contextlib.suppress(FileNotFoundError):
+            os.remove(old)
     inc = [*cpp_extension.include_paths("cuda"), "/usr/local/cuda/include", sysconfig.get_path("include")]
     lib = os.path.join(os.path.dirname(torch.__file__), "lib")
     tmp = FRONT + f".tmp{os.getpid()}"
@@ -68,6 +89,9 @@ def build_front(force=False):
     if r.returncode != 0:
         raise RuntimeError(f"g++ failed on front.cpp:\n{r.stdout}\n{r.stderr}")
     os.replace(tmp, FRONT)
+    with open(FRONT_STAMP + f".tmp{os.getpid()}", "w") as f:
+        f.write(front_built_against())
+    os.replace(f.name, FRONT_STAMP)
     return FRONT
 
 
