@@ -148,21 +148,27 @@ __device__ __forceinline__ void solve_cell(const EmitReq &q, int64_t cell, int l
     Pow2 ns = pow2_pair(-mc);
     float ah = 0.f, al = 0.f;  // absorbed power n 2^-m_c Pe 2^-Eg, float-float
     for (int gb = 0; gb < G8; gb += 32 * NB) {
-        int gi[NB], fl[NB];
-        float s[NB], nv[NB], Tv[NB];
-        float4 gq[NB];
+        float s[NB], nv[NB];
         if (gb == 0) {
 #pragma unroll
             for (int i = 0; i < NB; ++i) { s[i] = s0[i]; nv[i] = n0[i]; }
         } else {
             load_pass<NB, TONLY>(q, cell, gb, lane, s, nv);
         }
+        // four grains at once are more than the emission kernels' 80 registers hold
+        // (24 bytes spilled; 131072 cells x 150 x 126, 12 + 12 warps: 545 us, in halves 531)
+        constexpr int H = NB == 4 && EMIT ? 2 : NB;
+        int gi[H];
+        float4 gq[H];
+        auto load_grains = [&](int h) {
 #pragma unroll
-        for (int i = 0; i < NB; ++i) {
-            const int g = gb + lane + 32 * i;
-            gi[i] = g < G ? g : 0;
-            gq[i] = __ldg(reinterpret_cast<const float4 *>(tb.gp) + gi[i]);
-        }
+            for (int i = 0; i < H; ++i) {
+                const int g = gb + lane + 32 * (h + i);
+                gi[i] = g < G ? g : 0;
+                gq[i] = __ldg(reinterpret_cast<const float4 *>(tb.gp) + gi[i]);
+            }
+        };
+        load_grains(0);
         if (one && emit && !mass) {
             float mx = 0.f;
 #pragma unroll
@@ -170,27 +176,35 @@ __device__ __forceinline__ void solve_cell(const EmitReq &q, int64_t cell, int l
             mc = warp_exponent(mx);
             ns = pow2_pair(-mc);
         }
-        solve_batch<NB>(tb, gi, s, gq, Tv, fl);
 #pragma unroll
-        for (int i = 0; i < NB; ++i) {
-            const int g = gb + lane + 32 * i;
-            if (g >= G8) continue;
-            float invT = PAD_INV_T, nn = 0.f;
-            if (g < G) {
-                if (store) {
-                    q.T[cell * G + g] = Tv[i];
-                    if (q.flags) q.flags[cell * G + g] = (uint8_t)fl[i];
+        for (int h = 0; h < NB; h += H) {
+            int fl[H];
+            float sh[H], Tv[H];
+            if (h) load_grains(h);
+#pragma unroll
+            for (int i = 0; i < H; ++i) sh[i] = s[h + i];
+            solve_batch<H>(tb, gi, sh, gq, Tv, fl);
+#pragma unroll
+            for (int i = 0; i < H; ++i) {
+                const int g = gb + lane + 32 * (h + i);
+                if (g >= G8) continue;
+                float invT = PAD_INV_T, nn = 0.f;
+                if (g < G) {
+                    if (store) {
+                        q.T[cell * G + g] = Tv[i];
+                        if (q.flags) q.flags[cell * G + g] = (uint8_t)fl[i];
+                    }
+                    if (!TONLY) grain_out(tb, g, Tv[i], fl[i], sh[i], nv[h + i], ns, mass, rs, invT, nn, ah, al);
                 }
-                if (!TONLY) grain_out(tb, g, Tv[i], fl[i], s[i], nv[i], ns, mass, rs, invT, nn, ah, al);
-            }
-            if (emit) {
-                if (SMEM && g < gsm) {
-                    if (mass) reinterpret_cast<float *>(spairs)[g] = invT;
-                    else spairs[g] = make_float2(invT, nn);
-                }
-                if (!SMEM || also_glb) {
-                    if (mass) reinterpret_cast<float *>(q.prep)[cell * G8 + g] = invT;
-                    else q.prep[cell * G8 + g] = make_float2(invT, nn);
+                if (emit) {
+                    if (SMEM && g < gsm) {
+                        if (mass) reinterpret_cast<float *>(spairs)[g] = invT;
+                        else spairs[g] = make_float2(invT, nn);
+                    }
+                    if (!SMEM || also_glb) {
+                        if (mass) reinterpret_cast<float *>(q.prep)[cell * G8 + g] = invT;
+                        else q.prep[cell * G8 + g] = make_float2(invT, nn);
+                    }
                 }
             }
         }
@@ -810,9 +824,9 @@ __device__ __forceinline__ void cell_resid(const EmitReq &q, int64_t cell) {
 // with these, once claims, tile numbers and tables no longer stood in the
 // items' way (0.91 ms before); without any solve 12, 16 and 20 emission warps
 // take 0.74, 0.70 and 0.69 ms, and fewer than 8 solver warps fall behind.
-constexpr int fe_w(bool pass) { return pass ? 12 : 16; }
-constexpr int fs_w(bool pass) { return pass ? 12 : 8; }
-constexpr int fse_th(bool pass) { return (fe_w(pass) + fs_w(pass)) * 32; }
+// Which role paces a tile depends on the shape, so the 24 are shared out by it
+// (fse_emission_warps).
+constexpr int FSE_W = 24, FSE_TH = FSE_W * 32;
 constexpr int FSE_NBUF = 3;  // pair-tile buffers: the solvers run up to FSE_NBUF tiles ahead
 constexpr int FSE_TC = 32;   // cells per tile: one per lane of an emission item
 
@@ -827,9 +841,9 @@ __device__ __forceinline__ int fse_tile(int it, int nb) {
     return (int)blockIdx.x + j * (int)gridDim.x;
 }
 
-template <int NB, bool MASS, bool PASS>
-__global__ void __launch_bounds__(fse_th(PASS), 1) k_solve_emit(const __grid_constant__ EmitReq q) {
-    constexpr int FE_W = fe_w(PASS), FS_W = fs_w(PASS), FSE_TH = fse_th(PASS);
+template <int NB, bool MASS, bool PASS, int FE_W>
+__global__ void __launch_bounds__(FSE_TH, 1) k_solve_emit(const __grid_constant__ EmitReq q) {
+    constexpr int FS_W = FSE_W - FE_W;
     let_next_kernel_start();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const DevTables &tb = q.tb;
@@ -1349,21 +1363,38 @@ size_t plan_solve_emit(const dust_ctx *ctx, bool emit, bool mass, int *TC, int *
 }
 
 // The fused kernel over one request (general form), then the residual fold.
-template <bool MASS, bool PASS>
+template <bool MASS, bool PASS, int FE_W>
 int launch_fse(const EmitReq &r, int nb, unsigned grid, size_t smem, bool early, cudaStream_t st) {
-    const void *kern = nb == 1 ? reinterpret_cast<const void *>(k_solve_emit<1, MASS, PASS>)
-                     : nb == 2 ? reinterpret_cast<const void *>(k_solve_emit<2, MASS, PASS>)
-                     : nb == 3 ? reinterpret_cast<const void *>(k_solve_emit<3, MASS, PASS>)
-                               : reinterpret_cast<const void *>(k_solve_emit<4, MASS, PASS>);
+    auto kern = nb == 1 ? k_solve_emit<1, MASS, PASS, FE_W> : nb == 2 ? k_solve_emit<2, MASS, PASS, FE_W>
+              : nb == 3 ? k_solve_emit<3, MASS, PASS, FE_W> : k_solve_emit<4, MASS, PASS, FE_W>;
     DUST_CUDA_TRY(allow_shared_memory(kern));
-    switch (nb) {
-        case 1: DUST_CUDA_TRY(launch_early(early, k_solve_emit<1, MASS, PASS>, grid, fse_th(PASS), smem, st, r)); break;
-        case 2: DUST_CUDA_TRY(launch_early(early, k_solve_emit<2, MASS, PASS>, grid, fse_th(PASS), smem, st, r)); break;
-        case 3: DUST_CUDA_TRY(launch_early(early, k_solve_emit<3, MASS, PASS>, grid, fse_th(PASS), smem, st, r)); break;
-        default: DUST_CUDA_TRY(launch_early(early, k_solve_emit<4, MASS, PASS>, grid, fse_th(PASS), smem, st, r)); break;
-    }
-    DUST_CUDA_TRY(cudaGetLastError());
+    DUST_CUDA_TRY(launch_early(early, kern, grid, FSE_TH, smem, st, r));
     return DUST_OK;
+}
+
+// Emission warps of a one-pass launch.  The emission of a tile is NKG groups of
+// eight wavelengths per group of eight grains; its solve, a latency-bound chain,
+// is worth 60 of these and 16 more per group of grains (40 more again with four
+// grains per lane).  Fitted to the best of 12, 14 and 16 emission warps at 180
+// shapes from 90 x 12 to 400 x 96, general and dust-mass form, 20011 and 131072
+// cells: 0.12 % from the best on average, 4 % at most.  With 16 + 8 for every
+// shape the solvers paced narrow grids.  131072 cells, us per call: 12 + 8 warps of 96
+// registers (the kernel before) / 16 + 8 / now: 100 x 96 390 / 383 / 347, 100 x 126
+// 490 / 521 / 455, 150 x 126 552 / 602 / 531, 180 x 126 617 / 647 / 606, 200 x 96 521 /
+// 485 / 485.
+int fse_emission_warps(const DevTables &tb) {
+    const int groups = tb.G8 / 8, emission = tb.NKG * groups;
+    const int solve = 60 + 16 * groups + (groups > 12 ? 40 : 0);
+    return emission < solve ? 12 : emission < solve + 12 + 2 * groups ? 14 : 16;
+}
+
+template <bool MASS>
+int launch_fse_split(const EmitReq &r, int nb, unsigned grid, size_t smem, bool early, cudaStream_t st) {
+    switch (fse_emission_warps(r.tb)) {
+        case 12: return launch_fse<MASS, false, 12>(r, nb, grid, smem, early, st);
+        case 14: return launch_fse<MASS, false, 14>(r, nb, grid, smem, early, st);
+        default: return launch_fse<MASS, false, 16>(r, nb, grid, smem, early, st);
+    }
 }
 
 // Small calls (k_solve_emit_split): lanes per cell, the parts a tile's k-groups
@@ -1438,16 +1469,17 @@ int launch_solve_emit_fused(const EmitReq &req, int TC, size_t smem, int num_sms
     E.ntiles = (r.C + TC - 1) / TC;
     // grains per lane and pass of the solver warps: a cell is one pass up to
     // 32 NB_MAX grains.  With grain passes the first launch solves every grain
-    // but emits only a chunk of them, so its solver warps are its critical
-    // role: more of them, and three grains per lane, where a fourth spills at
-    // their 80 registers (131072 cells x 500 x 240: 3.01 ms per step with 12 +
-    // 12 warps and three, 3.03 with four, 3.05 with 12 + 8 warps and four).
+    // but emits only a chunk of them, so its solver warps are its critical role:
+    // 12 of them, and three grains per lane, or four where that is a pass less for up
+    // to 256 grains (65536 cells, us with three and four: 400 x 114 753 and 735, 500
+    // x 240 1590 and 1577, 200 x 360 1232 and 1238, 300 x 480 2234 and 2258).
     const bool pass = r.g1 - r.g0 < r.tb.G8;  // the first of several grain passes
-    const int nb = std::min(pass ? 3 : NB_MAX, (r.tb.G8 + 31) / 32);
+    const int G8 = r.tb.G8;
+    const int nb = G8 <= 96 ? (G8 + 31) / 32 : !pass || (G8 <= 256 && (G8 + 127) / 128 < (G8 + 95) / 96) ? 4 : 3;
     const bool mass = (r.mode & EMIT_MASS) != 0;
     const unsigned grid = (unsigned)std::min<int64_t>(E.ntiles, num_sms);
-    int rc = mass ? (pass ? launch_fse<true, true>(r, nb, grid, smem, early, st) : launch_fse<true, false>(r, nb, grid, smem, early, st))
-                  : (pass ? launch_fse<false, true>(r, nb, grid, smem, early, st) : launch_fse<false, false>(r, nb, grid, smem, early, st));
+    int rc = mass ? (pass ? launch_fse<true, true, 12>(r, nb, grid, smem, early, st) : launch_fse_split<true>(r, nb, grid, smem, early, st))
+                  : (pass ? launch_fse<false, true, 12>(r, nb, grid, smem, early, st) : launch_fse_split<false>(r, nb, grid, smem, early, st));
     if (rc != DUST_OK) return rc;
     if (nlaunch) *nlaunch = 1;  // the residual fold runs inside the kernel
     return DUST_OK;
