@@ -335,7 +335,7 @@ cudaError_t allow_shared_memory(Kernel *kernel) {
 // its rings leave; the solves want more (262144 x 200 x 96: 919 us per step
 // plainly launched, 1002 early; temperatures only 211, 306).  They start early in calls
 // where the launch latency saved counts for more (early_solve; 16384 cells 105
-// -> 94 us, 32768 157 -> 154, 65536 274 -> 285).
+// -> 94 us, 32768 157 -> 154, 65536 274 -> 285; early_k_solve).
 template <class... P, class... A>
 cudaError_t launch_early(bool early, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
                          const A &...args) {
@@ -352,6 +352,15 @@ cudaError_t launch_early(bool early, void (*kernel)(P...), unsigned grid, unsign
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 inline bool early_solve(int64_t cells, int num_sms, bool tc) { return !tc || cells <= 256 * (int64_t)num_sms; }
+// The solve that is a kernel of its own lives on L1 (every SM reads every grain's
+// table) and stays beside the GEMM only while it is short: up to 6528 roots per SM,
+// counting 102 grains at most.  Temperatures only, us, early and plainly: 200 x
+// 12, 25000 cells 16.5 / 18.5; 200 x 48, 20011 cells 22.6 / 22.6, 36000 28.8 / 26.7;
+// 200 x 96, 8192 cells 16.4 / 17.9, 16384 24.7 / 24.6, 20011 30.8 / 26.7, 32768 39.5 /
+// 30.8; 300 x 240, 8192 cells 30.8 / 32.8, 16384 42.1 / 42.3.
+inline bool early_k_solve(int64_t cells, int G, int num_sms, bool tc) {
+    return !tc || (early_solve(cells, num_sms, tc) && cells * (G < 102 ? G : 102) <= 6528 * (int64_t)num_sms);
+}
 __device__ __forceinline__ void after_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_next_kernel_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -169,7 +169,7 @@ int solve_view(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t 
         nl_total += nl;
         B.req[0].order = sv.order;
     }
-    const bool early = early_solve(C, ctx->num_sms, precision != DUST_PREC_FP32);
+    const bool tc = precision != DUST_PREC_FP32;
     if (rc == DUST_OK) {
         if (ev && ev[1]) DUST_CUDA_TRY(cudaEventRecord(ev[1], st));
         int nl = 0;
@@ -181,14 +181,15 @@ int solve_view(dust_ctx *ctx, int precision, int64_t C, const float *J, int64_t 
             // the solve runs inside the emission kernel: its time is reported with the emission's;
             // where the grains come in passes the kernel emits the first and k_emit the others
             if (ev && ev[2]) DUST_CUDA_TRY(cudaEventRecord(ev[2], st));
-            rc = launch_solve_emit_fused(B.req[0], ftc, fsmem, ctx->num_sms, st, &nl, early);
+            rc = launch_solve_emit_fused(B.req[0], ftc, fsmem, ctx->num_sms, st, &nl, early_solve(C, ctx->num_sms, tc));
             if (rc == DUST_OK && fgc < (mass ? ctx->tbm : ctx->tb).G8) {
                 nl_total += nl;
                 nl = 0;
                 rc = launch_emit_batch(B, ctx->num_sms, st, nullptr, true, &nl, 1);
             }
         } else {
-            rc = launch_emit_batch(B, ctx->num_sms, st, ev ? ev[2] : nullptr, fused, &nl, 0, early);
+            rc = launch_emit_batch(B, ctx->num_sms, st, ev ? ev[2] : nullptr, fused, &nl, 0,
+                                   early_k_solve(C, ctx->G, ctx->num_sms, tc));
         }
         nl_total += nl;
         if (ev && ev[3]) DUST_CUDA_TRY(cudaEventRecord(ev[3], st));
