@@ -604,7 +604,10 @@ __device__ __forceinline__ void emit_item_out(const EmitReq &q, int64_t cell, in
 // 512 threads of 128 registers); with MANY 23 that claim the next one while
 // they emit one (768 threads of 80).  MANY needs tiles of at least as many
 // items as its warps hold, 46: with fewer, items claimed and not yet begun
-// keep the three buffers from being refilled.  Whole solves in two kernels, 15
+// keep the three buffers from being refilled; and units of more tiles than
+// buffers: in a shorter one the 15 with their 128 registers are ahead (600 x
+// 300, us with 15 and 23: 10000 cells 824 and 842, 20011 1217 and 1235, 32768
+// 1591 and 1590, 65536 2641 and 2595).  Whole solves in two kernels, 15
 // and 23: 200 x 96 (25 items) 262144 cells 1.20 and 1.60 ms, 350 x 96 (44)
 // 65536 cells 0.530 and 0.544, 500 x 240 (63) 65536 cells 1.718 and 1.694;
 // 131072 cells 500 x 240, of which these are the later grain passes, 3.03 and
@@ -1268,7 +1271,7 @@ int launch_emit_batch(EmitBatch &B, int num_sms, cudaStream_t st, cudaEvent_t be
                 units += ((E.req[k].C + KE_TC - 1) / KE_TC + tpu - 1) / tpu;
             }
             E.ntiles = tiles;
-            bool many = true;  // every request's tiles have the items that 23 warps hold
+            bool many = tpu > KE_NBUF;  // and every request's tiles have the items that 23 warps hold
             for (int k = 0; k < E.nreq; ++k) many = many && E.req[k].tb.NKG >= 2 * KE_MANY;
             auto kern = mass ? (many ? k_emit<true, true> : k_emit<true, false>)
                              : (many ? k_emit<false, true> : k_emit<false, false>);
