@@ -1365,6 +1365,29 @@ size_t plan_solve_emit(const dust_ctx *ctx, bool emit, bool mass, int *TC, int *
     return smem;
 }
 
+// The work of a tile's two roles in the fused kernel, in groups of eight wavelengths
+// by eight grains: the emission has NKG per eight grains; the solve, a latency-bound
+// chain, is worth 60 of them and 16 more per eight grains (40 more again with four
+// grains per lane).  Fitted with fse_emission_warps to the best of 12, 14 and 16
+// emission warps at 180 shapes from 90 x 12 to 400 x 96, general and dust-mass
+// form, 20011 and 131072 cells: 0.12 % from the best on average, 4 % at most.
+struct FusedWork {
+    int emission, solve;
+};
+FusedWork fused_work(const DevTables &tb) {
+    const int groups = tb.G8 / 8;
+    return {tb.NKG * groups, 60 + 16 * groups + (groups > 12 ? 40 : 0)};
+}
+
+// Emission warps of a one-pass launch.  With 16 + 8 for every shape the solvers paced
+// narrow grids.  131072 cells, us per call: 12 + 8 warps of 96 registers (the kernel
+// before) / 16 + 8 / now: 100 x 96 390 / 383 / 347, 100 x 126 490 / 521 / 455, 150 x 126
+// 552 / 602 / 531, 180 x 126 617 / 647 / 606, 200 x 96 521 / 485 / 485.
+int fse_emission_warps(const DevTables &tb) {
+    const FusedWork w = fused_work(tb);
+    return w.emission < w.solve ? 12 : w.emission < w.solve + 12 + tb.G8 / 4 ? 14 : 16;
+}
+
 // The fused kernel over one request (general form), then the residual fold.
 template <bool MASS, bool PASS, int FE_W>
 int launch_fse(const EmitReq &r, int nb, unsigned grid, size_t smem, bool early, cudaStream_t st) {
@@ -1373,22 +1396,6 @@ int launch_fse(const EmitReq &r, int nb, unsigned grid, size_t smem, bool early,
     DUST_CUDA_TRY(allow_shared_memory(kern));
     DUST_CUDA_TRY(launch_early(early, kern, grid, FSE_TH, smem, st, r));
     return DUST_OK;
-}
-
-// Emission warps of a one-pass launch.  The emission of a tile is NKG groups of
-// eight wavelengths per group of eight grains; its solve, a latency-bound chain,
-// is worth 60 of these and 16 more per group of grains (40 more again with four
-// grains per lane).  Fitted to the best of 12, 14 and 16 emission warps at 180
-// shapes from 90 x 12 to 400 x 96, general and dust-mass form, 20011 and 131072
-// cells: 0.12 % from the best on average, 4 % at most.  With 16 + 8 for every
-// shape the solvers paced narrow grids.  131072 cells, us per call: 12 + 8 warps of 96
-// registers (the kernel before) / 16 + 8 / now: 100 x 96 390 / 383 / 347, 100 x 126
-// 490 / 521 / 455, 150 x 126 552 / 602 / 531, 180 x 126 617 / 647 / 606, 200 x 96 521 /
-// 485 / 485.
-int fse_emission_warps(const DevTables &tb) {
-    const int groups = tb.G8 / 8, emission = tb.NKG * groups;
-    const int solve = 60 + 16 * groups + (groups > 12 ? 40 : 0);
-    return emission < solve ? 12 : emission < solve + 12 + 2 * groups ? 14 : 16;
 }
 
 template <bool MASS>
@@ -1411,11 +1418,19 @@ SplitPlan plan_solve_emit_split(const dust_ctx *ctx, int64_t C, bool mass) {
     // but wants whole tiles for every SM.  Times per call of the fused kernel
     // and of this one, in us: 200 x 96, 7000 cells 64 / 61, 8192 64 / 65; 350 x
     // 96, 7000 cells 88 / 98, 8192 89 / 123; 64 x 16, 9728 cells 38 / 22, 12288
-    // 43 / 29.  Where its weights need grain passes (500 x 240) this one, which
-    // splits them by wavelength, stays ahead longer: 7000 cells 357 / 318, 8192
-    // 363 / 365, 9728 370 / 425.
+    // 43 / 29.  Where its weights need grain passes this one stays ahead longer,
+    // 300 x 126, 7296 cells 129 / 111, 7904 129 / 138; 200 x 240, 6688 cells 174 / 140,
+    // 7904 176 / 177.  With more than 128 grains, which take several passes of the
+    // solve in every part of a tile, and an emission well above the solve
+    // (fse_emission_warps), the fused form is ahead again near the end of its first
+    // round of tiles and from the middle of the second on: 500 x 240, 4408 cells 241 / 234,
+    // 4864 242 / 253, 6688 334 / 329, 7904 342 / 380; 600 x 480, 4864 cells 550 / 619, 6688
+    // 814 / 834, 7904 826 / 981; 350 x 180, 4864 cells 152 / 160, 6080 200 / 189, 7296 202 /
+    // 218.
     const bool passes = plan_emit(ctx, true, mass).gcp < tb.G8;
     if (C > 32 * sms && (passes ? C > 52 * sms : C > 96 * sms || (double)C * tb.K * tb.G > 1.4e8)) return p;
+    const FusedWork w = fused_work(tb);
+    if (passes && tb.G8 > 128 && 2 * w.emission > 3 * w.solve && (C > 44 * sms || (C > 28 * sms && C <= 32 * sms))) return p;
     // Four lanes per cell while tiles of 8 cells make at most two CTAs per SM, the
     // most that run at once; then two.  (200 x 96, in us with 1, 2 and 4 lanes: 32
     // cells 35 / 29 / 25, 1024 cells 39 / 35 / 31, 2048 cells 49 / 39 / 37, 4864
