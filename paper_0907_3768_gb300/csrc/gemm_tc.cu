@@ -249,7 +249,7 @@ __device__ __forceinline__ void solve_row(const EmitReq &q, int64_t cell, bool v
                 for (int i = 0; i < 4; ++i) nv[i] = g0 + i < G ? __ldg(nrow + g0 + i) : 0.f;
             }
         }
-        solve_batch<4>(tb, gi, sv, gq, Tv, fl);
+        solve_batch<4, true>(tb, gi, sv, gq, Tv, fl);
         if (!valid) continue;
         if (tvec && full) {
             *reinterpret_cast<float4 *>(Trow + g0) = make_float4(Tv[0], Tv[1], Tv[2], Tv[3]);

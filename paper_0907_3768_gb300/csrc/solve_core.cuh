@@ -50,10 +50,17 @@ __device__ __forceinline__ float hermite(float p0, float d0, float p1, float d1,
 // float's own bits (adding 2^23): the conversion instructions run on the same
 // quarter-rate pipe as the emission's ex2, and each costs its latency in a
 // chain that is all latency.
-template <int NB>
+// ROW: one thread takes a cell's grains in series (the absorption kernel's
+// epilogue).  There nothing else wants the conversion pipe, and the plain
+// conversions, all table loads behind one another and the root's steps as a loop
+// are ahead: temperatures only, 200 x 96, us with the forms of the other kernels and
+// with these: BF16 20011 cells 44.8 and 43.1, FP16 20011 49.1 and 47.3, 1024 41.0 and
+// 39.0.  The values are the same.
+template <int NB, bool ROW = false>
 __device__ __forceinline__ void solve_batch(const DevTables &tb, const int (&g)[NB], const float (&s)[NB],
                                             const float4 (&gq)[NB], float (&T)[NB], int (&fl)[NB]) {
     float ty[NB];
+    int at[ROW ? NB : 1];  // (ROW: the intervals)
     float4 rv[NB];
     const float mmax = (float)(tb.NI - 2);
 #pragma unroll
@@ -64,7 +71,7 @@ __device__ __forceinline__ void solve_batch(const DevTables &tb, const int (&g)[
         const int bits = __float_as_int(s[i]);
         const bool pos = s[i] > 0.f;  // false for 0, negatives and NaN
         // exponent field - 126, exactly: (2^23 + field) - (2^23 + 126)
-        const float ef = __int_as_float(0x4b000000 | ((bits >> 23) & 0xff)) - 8388734.f;
+        const float ef = ROW ? (float)(((bits >> 23) & 0xff) - 126) : __int_as_float(0x4b000000 | ((bits >> 23) & 0xff)) - 8388734.f;
         const float Y0 = pos ? ef + gq[i].x : 0.f;
         const float ly = pos ? lg2_approx(__int_as_float((bits & 0x007fffff) | 0x3f000000)) : 0.f;
         const float y = pos ? Y0 + ly : -INFINITY;
@@ -76,12 +83,21 @@ __device__ __forceinline__ void solve_batch(const DevTables &tb, const int (&g)[
         // instead of ~2^-24 of y invdy (a few thousand)
         const float ah = Y0 * gq[i].z, al = fmaf(Y0, gq[i].z, -ah), b = ly * gq[i].z;
         // m = floor of the coordinate clamped to [0, NI - 2], by a downward-rounded sum with 2^23
-        const float fm = __fadd_rd(fminf(fmaxf(ah + b, 0.f), mmax), 8388608.f);
-        const unsigned m = (unsigned)__float_as_int(fm) & 0x7fffffu;
-        ty[i] = fminf(fmaxf(((ah - (fm - 8388608.f)) + b) + al, 0.f), 1.f);
-        // byte offset below 2^30 (G <= 512, NI <= 65536): 32-bit arithmetic
-        rv[i] = __ldg(reinterpret_cast<const float4 *>(reinterpret_cast<const char *>(tb.ivr) +
-                                                       ((unsigned)g[i] * (unsigned)(tb.NI - 1) + m) * 16u));
+        if constexpr (ROW) {
+            at[i] = min(max((int)floorf(ah + b), 0), tb.NI - 2);
+            ty[i] = fminf(fmaxf(((ah - (float)at[i]) + b) + al, 0.f), 1.f);
+        } else {
+            const float fm = __fadd_rd(fminf(fmaxf(ah + b, 0.f), mmax), 8388608.f);
+            const unsigned m = (unsigned)__float_as_int(fm) & 0x7fffffu;
+            ty[i] = fminf(fmaxf(((ah - (fm - 8388608.f)) + b) + al, 0.f), 1.f);
+            // byte offset below 2^30 (G <= 512, NI <= 65536): 32-bit arithmetic
+            rv[i] = __ldg(reinterpret_cast<const float4 *>(reinterpret_cast<const char *>(tb.ivr) +
+                                                           ((unsigned)g[i] * (unsigned)(tb.NI - 1) + m) * 16u));
+        }
+    }
+    if constexpr (ROW) {
+#pragma unroll
+        for (int i = 0; i < NB; ++i) rv[i] = __ldg(tb.ivr + (size_t)g[i] * (tb.NI - 1) + at[i]);
     }
     // 2^x = sum_n (x ln 2)^n / n!, five terms: |x| <= 1/8 leaves < 6e-10 (tables
     // with a wider interval take ex2)
@@ -98,18 +114,32 @@ __device__ __forceinline__ void solve_batch(const DevTables &tb, const int (&g)[
         // term alone, so it carries no cancellation.
         const float d0 = rv[i].z, d1 = rv[i].w;
         const float c2 = -2.f * d0 - d1, c3 = d0 + d1;
-        float t = ty[i];
-        const float q = t * (d0 + t * (c2 + t * c3));
-        const float dq = 1.f + d0 + t * (2.f * c2 + 3.f * t * c3);
-        float nt = t - q * rcp_approx(dq);
-        const float lo = q < 0.f ? t : 0.f, hi = q < 0.f ? 1.f : t;
-        if (!(nt >= lo && nt <= hi)) {  // rare: bisect, then one more step
-            t = 0.5f * (lo + hi);
-            const float q2 = (t - ty[i]) + t * (d0 + t * (c2 + t * c3));
-            const float dq2 = 1.f + d0 + t * (2.f * c2 + 3.f * t * c3);
-            const float lo2 = q2 < 0.f ? t : lo, hi2 = q2 < 0.f ? hi : t;
-            nt = t - q2 * rcp_approx(dq2);
-            if (!(nt >= lo2 && nt <= hi2)) nt = 0.5f * (lo2 + hi2);
+        float t = ty[i], nt;
+        if constexpr (ROW) {
+            float lo = 0.f, hi = 1.f;
+            for (int it = 0; it < 2; ++it) {
+                const float q = (t - ty[i]) + t * (d0 + t * (c2 + t * c3));
+                const float dq = 1.f + d0 + t * (2.f * c2 + 3.f * t * c3);
+                lo = q < 0.f ? t : lo;
+                hi = q < 0.f ? hi : t;
+                nt = t - q * rcp_approx(dq);
+                const bool inside = nt >= lo && nt <= hi;
+                t = nt = inside ? nt : 0.5f * (lo + hi);
+                if (inside) break;
+            }
+        } else {
+            const float q = t * (d0 + t * (c2 + t * c3));
+            const float dq = 1.f + d0 + t * (2.f * c2 + 3.f * t * c3);
+            nt = t - q * rcp_approx(dq);
+            const float lo = q < 0.f ? t : 0.f, hi = q < 0.f ? 1.f : t;
+            if (!(nt >= lo && nt <= hi)) {  // rare: bisect, then one more step
+                t = 0.5f * (lo + hi);
+                const float q2 = (t - ty[i]) + t * (d0 + t * (c2 + t * c3));
+                const float dq2 = 1.f + d0 + t * (2.f * c2 + 3.f * t * c3);
+                const float lo2 = q2 < 0.f ? t : lo, hi2 = q2 < 0.f ? hi : t;
+                nt = t - q2 * rcp_approx(dq2);
+                if (!(nt >= lo2 && nt <= hi2)) nt = 0.5f * (lo2 + hi2);
+            }
         }
         // T = 2^u_m 2^(tau du)
         const float x = nt * rv[i].y;
