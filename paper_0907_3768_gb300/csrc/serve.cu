@@ -183,6 +183,10 @@ void finish_req(dust_server *s, ServeReq *r, int state, int status) {
     }
 }
 
+// Whether nothing of a request is on the GPU or with the scheduler any more: a failed
+// or cancelled one keeps its footprint until its last part has retired.
+bool finished(const ServeReq *r) { return r->state == RS_DONE || ((r->state == RS_CANCELLED || r->state == RS_FAILED) && !r->footprint); }
+
 void admit(dust_server *s) {
     for (auto it = s->queue.begin(); it != s->queue.end();) {
         ServeReq *r = *it;
@@ -576,8 +580,8 @@ int dust_serve_poll(dust_server *s, uint64_t ticket, int *state, double *latency
     auto it = s->by_ticket.find(ticket);
     if (it == s->by_ticket.end()) return set_error(DUST_ENOTFOUND, "unknown ticket %llu", (unsigned long long)ticket);
     ServeReq *r = it->second;
-    const bool fin = r->state == RS_DONE || r->state == RS_CANCELLED || (r->state == RS_FAILED && !r->footprint);
-    if (state) *state = fin ? r->state : (r->state == RS_FAILED ? RS_ACTIVE : r->state);
+    const bool fin = finished(r);
+    if (state) *state = fin ? r->state : r->state == RS_QUEUED ? RS_QUEUED : RS_ACTIVE;
     if (latency_ms) *latency_ms = fin ? r->t_done - r->t_submit : now_ms() - r->t_submit;
     if (fin) {
         const int st = r->state, status = r->status;
@@ -597,7 +601,7 @@ int dust_serve_wait(dust_server *s, uint64_t ticket, double timeout_ms, double *
         if (it == s->by_ticket.end())
             return set_error(DUST_ENOTFOUND, "unknown ticket %llu", (unsigned long long)ticket);
         ServeReq *r = it->second;
-        const bool fin = r->state == RS_DONE || r->state == RS_CANCELLED || (r->state == RS_FAILED && !r->footprint);
+        const bool fin = finished(r);
         if (fin) {
             if (latency_ms) *latency_ms = r->t_done - r->t_submit;
             const int st = r->state, status = r->status;
