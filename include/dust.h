@@ -256,7 +256,8 @@ int dust_ctx_profile_read(dust_ctx *ctx, double *ms_absorb, double *ms_solve, do
  * large ones not starved); small ones go whole into batched rounds (one
  * launch per kernel for up to 32 of them), large ones run alone a chunk at a
  * time through dust_solve's path.  Requests arriving while the GPU is busy
- * join a round as soon as one retires.  A request's results are bitwise
+ * join a round as soon as one retires (a batched round that is not full waits
+ * for a short one before it to retire).  A request's results are bitwise
  * those of dust_solve on the same context with the context's precision at
  * submit time.  The paper
  * processes one grid per call (Section 5); serving has no counterpart there.
@@ -277,7 +278,8 @@ int dust_ctx_profile_read(dust_ctx *ctx, double *ms_absorb, double *ms_solve, do
  * dust_serve_wait: blocks up to timeout_ms; DUST_ETIMEOUT if still running,
  * DUST_OK when done (ticket released).
  * dust_serve_cancel: a queued request is dropped; an active one gets no
- * further chunks (chunks already launched finish; its outputs are partial).
+ * further chunks (chunks already launched finish; its outputs are partial, and
+ * it counts as active until the last of them has).
  * dust_server_destroy: cancels queued requests, finishes active ones, frees
  * everything. */
 typedef struct {

@@ -8,7 +8,8 @@
 // from a first-fit arena carved out of one allocation.  Work proceeds in
 // rounds, two in flight, so requests that arrive while the GPU is busy join a
 // round as soon as one retires and their work overlaps with the tail of
-// earlier ones.  Rounds are sized by work, shortest remaining first: active
+// earlier ones (a batched round that could still grow waits for a short one to
+// retire).  Rounds are queued without the server's lock.  Rounds are sized by work, shortest remaining first: active
 // requests are ranked by their remaining Planck terms discounted by how long
 // they have waited (so that large requests are not starved).  A small first
 // request (little work left) makes a batched round: it and the next small
@@ -104,6 +105,7 @@ struct Part {
 struct Round {
     cudaEvent_t ev = nullptr;
     int slot = 0;  // its part of the server's class-count workspace
+    double terms = 0.0;  // its Planck terms
     std::vector<Part> parts;
 };
 
@@ -213,7 +215,9 @@ void admit(dust_server *s) {
 // it and the next small ones whole, up to batch_terms and MAXREQ parts, for
 // the batched kernels; otherwise it takes a chunk of about chunk_terms of the
 // first alone (a multiple of 128 cells, at least 4096), for dust_solve's path.
-std::vector<Part> build_round(dust_server *s) {
+// gather: a short round is on the GPU, so a batched one that is not full yet is
+// left to grow until that one has retired.
+std::vector<Part> build_round(dust_server *s, bool gather) {
     std::vector<Part> parts;
     std::vector<std::pair<double, ServeReq *>> cand;
     const double t = now_ms();
@@ -227,15 +231,20 @@ std::vector<Part> build_round(dust_server *s) {
     ServeReq *top = cand[0].second;
     if (terms(top) <= s->small_terms) {
         double sum = 0.0;
+        bool full = false;
         for (const auto &c : cand) {
             ServeReq *r = c.second;
             const double w = terms(r);
-            if (w > s->small_terms || (!parts.empty() && sum + w > s->batch_terms)) continue;
+            if (w > s->small_terms) continue;
+            if ((full = parts.size() == (size_t)MAXREQ)) break;
+            if (!parts.empty() && sum + w > s->batch_terms) { full = true; continue; }
             parts.push_back({r, r->next, r->C - r->next});
-            r->next = r->C;
-            r->inflight_parts++;
             sum += w;
-            if (parts.size() == (size_t)MAXREQ) break;
+        }
+        if (gather && !full) return {};
+        for (const Part &p : parts) {
+            p.r->next = p.r->C;
+            p.r->inflight_parts++;
         }
         return parts;
     }
@@ -268,7 +277,11 @@ ScratchView part_view(const dust_server *s, const Part &p, int slot, int k) {
     return w;
 }
 
-int launch_round(dust_server *s, const Round &rd) {
+// Queues a round's kernels; counts them in *launches.  Runs without the server's
+// lock: of the server it reads what never changes (stream, limits, workspaces),
+// of the requests what their submission and admission fixed, and `ready`, which
+// while a request has parts in flight only this thread touches.
+int launch_round(const dust_server *s, const Round &rd, int64_t *launches) {
     const std::vector<Part> &parts = rd.parts;
     // a request's first round waits (on the device) for the work its
     // producer had queued before submitting
@@ -289,7 +302,7 @@ int launch_round(dust_server *s, const Round &rd) {
         const int rc = solve_view(r->ctx, r->precision, p.cn, r->J + p.c0 * r->ld, r->ld, r->n + p.c0 * G,
                                   r->T + p.c0 * G, r->L ? r->L + p.c0 * r->ld : nullptr, r->resid ? r->resid + p.c0 : nullptr,
                                   r->flags ? r->flags + p.c0 * G : nullptr, part_view(s, p, rd.slot, 0), s->st, false, &nl);
-        s->launches += (uint64_t)nl;
+        *launches += nl;
         return rc;
     }
     // absorption GEMMs, one launch per precision
@@ -307,7 +320,7 @@ int launch_round(dust_server *s, const Round &rd) {
             if (B.nreq) {
                 int rc = launch_simt_batch(B, s->st);
                 if (rc != DUST_OK) return rc;
-                s->launches++;
+                ++*launches;
             }
         } else {
             // one launch per orientation, each request in the one dust_solve uses for
@@ -337,7 +350,7 @@ int launch_round(dust_server *s, const Round &rd) {
                     int rc = finish_tc_batch(B, prec, s->smem_optin, &smem);
                     if (rc == DUST_OK) rc = launch_tc_batch(B, prec, smem, s->num_sms, s->st);
                     if (rc != DUST_OK) return rc;
-                    s->launches++;
+                    ++*launches;
                 }
             }
         }
@@ -372,11 +385,11 @@ int launch_round(dust_server *s, const Round &rd) {
     if (ob.nreq) {
         int rc = launch_order(ob, s->st, &nl);
         if (rc != DUST_OK) return rc;
-        s->launches += (uint64_t)nl;
+        *launches += nl;
     }
     int rc = launch_emit_batch(E, s->num_sms, s->st, nullptr, false, &nl);
     if (rc != DUST_OK) return rc;
-    s->launches += (uint64_t)nl;
+    *launches += nl;
     return DUST_OK;
 }
 
@@ -413,20 +426,33 @@ void scheduler(dust_server *s) {
         }
         admit(s);
         if (s->inflight.size() < (size_t)NSLOT) {
-            std::vector<Part> parts = build_round(s);
+            std::vector<Part> parts = build_round(s, !s->inflight.empty() && s->inflight.back().terms < s->batch_terms);
             if (!parts.empty()) {
                 Round rd;
+                for (const Part &q : parts) rd.terms += (double)q.cn * q.r->ctx->K * q.r->ctx->G;
                 if (!s->ev_pool.empty()) { rd.ev = s->ev_pool.back(); s->ev_pool.pop_back(); }
                 else cudaEventCreateWithFlags(&rd.ev, cudaEventDisableTiming);
                 rd.parts = std::move(parts);
                 while (s->slot_busy[rd.slot]) ++rd.slot;  // a free slot exists: fewer than NSLOT in flight
                 s->slot_busy[rd.slot] = true;
-                int rc = launch_round(s, rd);
-                if (rc == DUST_OK && cudaEventRecord(rd.ev, s->st) == cudaSuccess) {
+                // Submissions go on while the round's kernels are queued (some 30 us),
+                // and requests gather while a short round runs: with the lock held and
+                // every round queued at once, a single request of a few cells, which
+                // takes the GPU less time than its launches take the host, left the
+                // next ones to rounds of one (30 requests of 300 cells, 64 x 24: 25
+                // rounds, 0.78 ms; now 8.7, 0.50; 30 of 64 cells, 200 x 96 0.49 and
+                // 0.45; either change alone gains nothing).
+                int64_t launches = 0;
+                lk.unlock();
+                int rc = launch_round(s, rd, &launches);
+                if (rc == DUST_OK && cudaEventRecord(rd.ev, s->st) != cudaSuccess) rc = DUST_ECUDA;
+                lk.lock();
+                s->launches += launches;
+                if (rc == DUST_OK) {
                     s->rounds++;
                     s->inflight.push_back(std::move(rd));
                 } else {
-                    retire_round(s, rd, rc == DUST_OK ? DUST_ECUDA : rc);
+                    retire_round(s, rd, rc);
                 }
                 continue;
             }
