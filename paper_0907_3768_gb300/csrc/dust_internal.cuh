@@ -394,7 +394,7 @@ int launch_tc_batch(const TcBatch &B, int precision, size_t smem, int num_sms, c
                     const SolveList *sl = nullptr);
 // FP32 SIMT batches.
 void make_simt_req(const dust_ctx *ctx, int64_t C, const float *J, int64_t ld, float *S, SimtReq &r);
-int launch_simt_batch(SimtBatch &B, cudaStream_t st);
+int launch_simt_batch(SimtBatch &B, int num_sms, cudaStream_t st);
 void fill_emit_req(const dust_ctx *ctx, const EmitPlan &p, int64_t C, const ScratchView &sv, const float *n,
                    float *T, float *L, int64_t ld, double *resid, uint8_t *flags, EmitReq &r, bool mass);
 // Numbers cells and tiles, then launches the solve over every request and the

@@ -318,7 +318,7 @@ int launch_round(const dust_server *s, const Round &rd, int64_t *launches) {
                 make_simt_req(r->ctx, p.cn, r->J + p.c0 * r->ld, r->ld, part_view(s, p, rd.slot, (int)k).S, B.req[B.nreq++]);
             }
             if (B.nreq) {
-                int rc = launch_simt_batch(B, s->st);
+                int rc = launch_simt_batch(B, s->num_sms, s->st);
                 if (rc != DUST_OK) return rc;
                 ++*launches;
             }
