@@ -17,8 +17,8 @@
 //   with a fresh quadrature per step (Section 4.3); the device table removes
 //   those exponentials.  Writes T, flags and, when the emission follows, the
 //   pairs (1/T, n 2^-m_c) and a per-cell record (m_c, absorbed power).
-// k_emit — persistent, one thread per (two cells, 8 consecutive wavelengths),
-//   Eq. 10:
+// k_emit — a CTA per work unit (a run of 32-cell tiles), one lane per cell and
+//   8 consecutive wavelengths, Eq. 10:
 //     L[c,k] = 2^(m_c+q_k) sum_g (n 2^-m_c) Chat[g,k] t/(1-t),
 //     t = 2^(nax_k / T[c,g])  (one MUFU ex2 per term),
 //   the grain sum accumulated as a fraction N/D over groups of 8 grains so
@@ -27,11 +27,9 @@
 //   Chat sits in shared memory ([k-group][grain][2] float4, odd row stride),
 //   in grain chunks when it does not fit, as the paper staged sigma per block
 //   (Section 4.4); the next tile's (1/T, n) pairs stream in with cp.async
-//   while the current tile computes.  Resident weights: two CTAs of 256
-//   threads per SM; streamed weights: one CTA of 512 threads, twice the cells
-//   per tile and nearly all of shared memory for the chunks.
+//   while the current tile computes.
 // k_solve_emit — one CTA per SM: solver warps run k_solve's per-cell code on
-//   the tile after the one being emitted and leave its pairs in shared
+//   the tiles ahead of the one being emitted and leave their pairs in shared
 //   memory; emission warps take one cell x 8 wavelengths per thread with
 //   k_emit's arithmetic.  The latency-bound solve hides behind the emission.
 // resid = sum_k w_k L[c,k] / (4 pi sum_g n Pe) - 1: both sums are kept in
@@ -532,10 +530,7 @@ __device__ __forceinline__ int64_t ordered_cell(const EmitReq &q, int64_t i) {
 
 
 // Epilogue of one emission item (one cell, the 8 wavelengths of k-group
-// ikg) in the warp-specialized kernel, the same arithmetic in the same order
-// as k_emit's inline epilogue (kept inline there: as a call it cost k_emit
-// 1-3 %): the accumulators scaled by
-// 2^(m_c + q_k) (times the cell's mass mantissa ms in the dust-mass form) are
+// ikg), for every emission kernel: the accumulators scaled by 2^(m_c + q_k) (times the cell's mass mantissa ms in the dust-mass form) are
 // stored as L, as two 16-byte stores (one 32-byte sector) when the row allows
 // it, and the item's residual partial sum_k w_k L_k is accumulated
 // error-free in float-float (products split by FMA, sums by two-sum).
@@ -829,6 +824,11 @@ __device__ __forceinline__ void cell_resid(const EmitReq &q, int64_t cell) {
 // take 0.74, 0.70 and 0.69 ms, and fewer than 8 solver warps fall behind.
 // Which role paces a tile depends on the shape, so the 24 are shared out by it
 // (fse_emission_warps).
+// Items are claimed ahead although a tile may have fewer of them than the warps
+// hold (k_emit's rule): with wide grids the counter's latency counts for more than a
+// buffer kept waiting.  131072 cells (262144 at 200 x 96), us claiming ahead and when an
+// item is begun: 350 x 96 831 / 841, 200 x 96 919 / 931, 150 x 126 531 / 536, 200 x 24 228 /
+// 228, 100 x 96 348 / 325, 64 x 96 281 / 272.
 constexpr int FSE_W = 24, FSE_TH = FSE_W * 32;
 constexpr int FSE_NBUF = 3;  // pair-tile buffers: the solvers run up to FSE_NBUF tiles ahead
 constexpr int FSE_TC = 32;   // cells per tile: one per lane of an emission item
