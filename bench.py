@@ -41,10 +41,10 @@ KERNEL_SOURCES = {
 }
 RECORDED_TRAFFIC = {
     # kernel: (bytes per launch on the bench's workload, profile summary, sources sha256[:16])
-    "k_solve_emit": (248.616192e6 + 361.798144e6, "profiles/k_solve_emit_2e18cells_K200_G96.md", "e3f7ff69c06fdd0b"),
-    "k_emit": (220.736256e6 + 218.525952e6, "profiles/k_emit_2e18cells_K200_G96.md", "e3f7ff69c06fdd0b"),
+    "k_solve_emit": (248.663552e6 + 361.792768e6, "profiles/k_solve_emit_2e18cells_K200_G96.md", "9d72c9ddbce265c0"),
+    "k_emit": (220.898816e6 + 219.147776e6, "profiles/k_emit_2e18cells_K200_G96.md", "9d72c9ddbce265c0"),
     # the full-size launch, DRAM counters only (one ncu pass; the 2^14-cell --set full capture is in the same file)
-    "k_fluct": (255.166208e6 + 175.692800e6, "profiles/k_fluct_2e14cells_K200_G36_M128.md", "b3d8c7bb4178b4a4"),
+    "k_fluct": (255.508480e6 + 175.476992e6, "profiles/k_fluct_2e14cells_K200_G36_M128.md", "8526c8114fc9db11"),
 }
 
 
