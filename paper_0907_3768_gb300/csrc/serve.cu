@@ -236,12 +236,14 @@ std::vector<Part> build_round(dust_server *s, bool gather) {
             ServeReq *r = c.second;
             const double w = terms(r);
             if (w > s->small_terms) continue;
-            if ((full = parts.size() == (size_t)MAXREQ)) break;
-            if (!parts.empty() && sum + w > s->batch_terms) { full = true; continue; }
+            if (parts.size() == (size_t)MAXREQ || (!parts.empty() && sum + w > s->batch_terms)) {
+                full = true;  // a smaller one may still fit
+                continue;
+            }
             parts.push_back({r, r->next, r->C - r->next});
             sum += w;
         }
-        if (gather && !full) return {};
+        if (gather && !full && parts.size() < (size_t)MAXREQ) return {};
         for (const Part &p : parts) {
             p.r->next = p.r->C;
             p.r->inflight_parts++;
